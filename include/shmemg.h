@@ -366,7 +366,8 @@ int shmemg_run_script_host(const shmemg_op_t *ops, int64_t nops, int64_t *fetche
 /* ----------------------------------------------------------------- AMO stress */
 /* Device-initiated AMO stream over an int64 table distributed across all PEs: word w
  * lives on PE w / words_per_pe at symmetric offset table + (w % words_per_pe) * 8.
- * One CTA per PE; PE p issues ops [p*nops/npes, (p+1)*nops/npes) in order.  Op i
+ * PE p's ops are [p*nops/npes, (p+1)*nops/npes); they are issued concurrently over the
+ * whole GPU (Sec. 6.3: atomicity does not imply ordering).  Op i
  * (packed uint32: bits 0..26 word, bits 27..28 code 0 fetch_add, 1 compare_swap,
  * 2 fetch_xor) takes r = splitmix64 counter draw (op_seed ^ i): fetch_add adds
  * (r mod 2^20) + 1, compare_swap swaps in r if the word equals its initial value

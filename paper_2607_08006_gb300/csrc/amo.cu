@@ -28,35 +28,49 @@ struct AmoArgs {
     uint8_t *state;       // reserved prefix (status word)
 };
 
-// One CTA per PE; PE p issues ops [p*nops/npes, (p+1)*nops/npes), a warp handles 32
-// consecutive ops per iteration (coalesced op reads and fetched writes).
-__global__ void __launch_bounds__(AMO_THREADS) k_amo_stream(AmoArgs a) {
+// A persistent grid cuts the stream into one contiguous range per CTA, in blocks of
+// AMO_THREADS ops (coalesced op reads and fetched writes).  Which PE an op is issued for
+// does not enter its result, so the PEs' ranges need no CTA of their own: one CTA per PE
+// left 88 of 152 SMs idle on a 64-PE heap (4 Mi random ops on a 128 MiB table: 294 us, now
+// 115; 1 Mi ops on an 8 MiB one: 45.1 us, now 12.3).  A random atomic is bound by
+// the rate of the table's sector fills and write-backs once enough are in flight, and more
+// lower it: with 6 CTAs per SM and 4 atomics per thread 4 Mi ops on a 512 MiB table ran
+// 150 us against 140 with 3 and 2 (the 128 MiB table 112 against 109; tables inside the L2
+// the same), so a plain stream runs AMO_PLAIN_CTAS CTAs per SM.  The aggregating form
+// has one pass of a warp in flight at a time and takes every CTA that fits (289 against
+// 284 us, 4 M Zipf ops).
+constexpr int AMO_U = 2;  // atomics in flight per thread
+constexpr int AMO_PLAIN_CTAS = 3;
+__global__ void __launch_bounds__(AMO_THREADS, 6) k_amo_stream(AmoArgs a) {
     __shared__ uint64_t s_val[AMO_THREADS];
     __shared__ uint64_t s_old[AMO_THREADS];
-    const int p = blockIdx.x;
-    const uint64_t lo = a.nops * (uint64_t)p / (uint64_t)a.npes;
-    const uint64_t hi = a.nops * (uint64_t)(p + 1) / (uint64_t)a.npes;
+    const uint64_t nblk = (a.nops + AMO_THREADS - 1) / AMO_THREADS;
+    const uint64_t lo = nblk * blockIdx.x / gridDim.x * AMO_THREADS, hi0 = nblk * (blockIdx.x + 1) / gridDim.x * AMO_THREADS;
+    const uint64_t hi = hi0 < a.nops ? hi0 : a.nops;
     if (!(a.flags & SHMEMG_AMO_AGGREGATE)) {
-        // each thread keeps four independent atomics in flight (ops i, i+B, i+2B, i+3B)
-        constexpr int U = 4;
-        for (uint64_t base = lo + threadIdx.x; base < hi; base += (uint64_t)blockDim.x * U) {
-            unsigned long long old[U];
-            bool act[U];
+        // each thread keeps AMO_U independent atomics in flight, their op words read first
+        for (uint64_t base = lo + threadIdx.x; base < hi; base += AMO_THREADS * AMO_U) {
+            uint32_t op[AMO_U];
+            unsigned long long old[AMO_U];
 #pragma unroll
-            for (int k = 0; k < U; k++) {
-                const uint64_t i = base + (uint64_t)k * blockDim.x;
-                act[k] = i < hi;
+            for (int k = 0; k < AMO_U; k++) {
+                const uint64_t i = base + (uint64_t)k * AMO_THREADS;
+                op[k] = i < hi ? __ldcs(a.ops + i) : 0u;
+            }
+            uint32_t act = 0;
+#pragma unroll
+            for (int k = 0; k < AMO_U; k++) {
+                const uint64_t i = base + (uint64_t)k * AMO_THREADS;
                 old[k] = 0;
-                if (!act[k]) continue;
-                const uint32_t op = __ldcs(a.ops + i);
-                const uint64_t w = op & ((1u << 27) - 1u);
-                const uint32_t code = (op >> 27) & 3u;
+                if (i >= hi) continue;
+                const uint64_t w = op[k] & ((1u << 27) - 1u);
+                const uint32_t code = (op[k] >> 27) & 3u;
                 if (w >= a.nwords || code == 3u) {
                     int *stw = (int *)(a.state + SHMEMG_STATUS_OFF);
                     if (atomicCAS(stw, 0, SHMEMG_ERR_INVALID_ARG) == 0) *(volatile int64_t *)(a.state + SHMEMG_STATUS_OFF + 8) = (int64_t)i;
-                    act[k] = false;
                     continue;
                 }
+                act |= 1u << k;
                 const uint64_t r = cb64(a.op_seed, i);
                 const uint64_t pe = a.wpp_log2 >= 0 ? w >> a.wpp_log2 : w / a.wpp;
                 const uint64_t idx = w - pe * a.wpp;
@@ -67,16 +81,17 @@ __global__ void __launch_bounds__(AMO_THREADS) k_amo_stream(AmoArgs a) {
             }
             if (a.fetched) {
 #pragma unroll
-                for (int k = 0; k < U; k++)
-                    if (act[k]) __stcs((unsigned long long *)a.fetched + base + (uint64_t)k * blockDim.x, old[k]);
+                for (int k = 0; k < AMO_U; k++)
+                    if (act >> k & 1u) __stcs((unsigned long long *)a.fetched + base + k * AMO_THREADS, old[k]);
             }
         }
         return;
     }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    // warp aggregation: a warp takes 32 consecutive ops per pass
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t lt = (1u << lane) - 1u;
     uint64_t *sv = s_val + warp * 32, *so = s_old + warp * 32;
-    for (uint64_t base = lo + (uint64_t)warp * 32; base < hi; base += (uint64_t)nwarps * 32) {
+    for (uint64_t base = lo + warp * 32; base < hi; base += AMO_THREADS) {
         const uint64_t i = base + lane;
         bool active = i < hi;
         uint32_t op = active ? __ldcs(a.ops + i) : 0u;
@@ -442,7 +457,12 @@ int shmemg_amo_stream(int64_t *table, uint64_t words_per_pe, const uint32_t *ops
         const uint64_t tiles = ((nops / S.npes + 1 + CB_TILE - 1) / CB_TILE) * S.npes;
         const int grid = (int)std::min<uint64_t>(tiles, (uint64_t)per_sm * S.sm_count);
         k_amo_combine<<<grid, CB_THREADS, CB_SMEM, to_stream(stream)>>>(a);
-    } else k_amo_stream<<<S.npes, AMO_THREADS, 0, to_stream(stream)>>>(a);
+    } else {
+        const uint64_t ctas = (nops + AMO_THREADS - 1) / AMO_THREADS;
+        const uint64_t cap = (flags & SHMEMG_AMO_AGGREGATE) ? (uint64_t)ctas_for((const void *)k_amo_stream, AMO_THREADS, 0)
+                                                            : (uint64_t)AMO_PLAIN_CTAS * (uint64_t)S.sm_count;
+        k_amo_stream<<<(unsigned)std::min(ctas, cap), AMO_THREADS, 0, to_stream(stream)>>>(a);
+    }
     return cuda_rc(cudaGetLastError());
 }
 
