@@ -423,10 +423,14 @@ int shmemg_pingpong_cluster(void *buf, uint64_t *sig, uint64_t payload, int npai
  *          rounded up to a multiple of 4 (work space: north and south rows, west and
  *          east columns, each part 16-byte aligned);
  *   sigs   4 uint64, zero before the call (left zero after a successful call).
+ * The other tile's contents after the call are unspecified.
  * shmemg_halo_jacobi: one cooperative launch; after each sweep a PE stores its new
  * boundary rows and columns straight into its four neighbours' halo buffers (device-
  * initiated puts fused into the sweep), then signals each neighbour (put-with-signal,
  * Sec. 7); before each sweep it waits for its four signals (bounded wait_until).
+ * Where a PE's tile fits the registers of its CTAs (up to 8 of
+ * them per PE, as the GPU holds at once) it stays there for the whole run and the boundary
+ * values travel as flagged words through the neighbours' tile 1; `halos` is then unused.
  * shmemg_halo_jacobi_plain: the same sweeps, one stream-ordered launch per sweep (the
  * plain launch-per-op path: kernel boundaries replace the signals).  tiles and halos
  * 16-byte aligned, px*py == npes, else SHMEMG_ERR_INVALID_ARG. */

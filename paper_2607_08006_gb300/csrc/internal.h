@@ -58,6 +58,10 @@ uint64_t balanced_grid(uint64_t nitems, uint64_t cap, int ngroups = 1);
 // (the interpreter's context agents: CTA npes + p serves PE p); SHMEMG_ERR_UNSUPPORTED if
 // the GPU cannot hold every CTA at once
 int launch_pe_grid(const void *kernel, void **args, size_t smem, cudaStream_t s, int threads = 0, int grid_mult = 1);
+// cooperative launch of `grid` CTAs in clusters of cluster_dim (1: none); with `query` only
+// whether the GPU can hold them all at once (SHMEMG_SUCCESS or SHMEMG_ERR_UNSUPPORTED)
+int launch_coop(const void *kernel, void **args, unsigned grid, int cluster_dim, int threads, size_t smem, cudaStream_t s,
+                bool query = false);
 int interp_threads();
 
 // splitmix64 (Steele, Lea, Flood, OOPSLA 2014): first output of the stream started at

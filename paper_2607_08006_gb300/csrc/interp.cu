@@ -765,10 +765,14 @@ int interp_threads() {
 // `threads` per CTA (0: the interpreter's count).
 int launch_pe_grid(const void *kernel, void **args, size_t smem, cudaStream_t s, int threads, int grid_mult) {
     State &S = st();
-    if (threads <= 0) threads = interp_threads();
-    const int cd = S.cluster_dim;
     const unsigned grid =
-        (S.pe_mode == SHMEMG_PE_MODE_CLUSTER ? (unsigned)(S.npes * cd) : (unsigned)S.npes) * (unsigned)grid_mult;
+        (S.pe_mode == SHMEMG_PE_MODE_CLUSTER ? (unsigned)(S.npes * S.cluster_dim) : (unsigned)S.npes) * (unsigned)grid_mult;
+    return launch_coop(kernel, args, grid, S.cluster_dim, threads > 0 ? threads : interp_threads(), smem, s);
+}
+
+int launch_coop(const void *kernel, void **args, unsigned grid, int cd, int threads, size_t smem, cudaStream_t s,
+                bool query) {
+    State &S = st();
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(threads);
@@ -817,6 +821,7 @@ int launch_pe_grid(const void *kernel, void **args, size_t smem, cudaStream_t s,
         }
     }
     if (!ok) return SHMEMG_ERR_UNSUPPORTED;
+    if (query) return SHMEMG_SUCCESS;
     cfg.attrs = attr;
     cfg.numAttrs = na;
     cudaError_t e = cudaLaunchKernelExC(&cfg, kernel, args);
