@@ -3,9 +3,10 @@
 // operation"): RMA, AMOs, put-with-signal, wait, and the team collectives, each one
 // full-grid kernel on the caller's stream.
 //
-// Data movement is split into work items of one chunk (blockDim x 4 vectors); a CTA
-// takes items round-robin, each thread keeps its 4 vector loads in flight before it
-// stores them (to one destination, or to every team member for broadcast/fcollect).
+// Data movement is split into work items: a chunk of one segment, shared by a group of
+// threads (a CTA, or a part of one where segments are small); each thread keeps up to four
+// 16-byte loads in flight before it stores them (to one destination, or to every team
+// member for broadcast/fcollect), whatever the segments' alignment and length.
 // Reductions use a slice-owner schedule: a thread owns a vector of elements, reads it
 // from every member, combines, and writes the result to every member.
 #include <cuda_runtime.h>
@@ -22,7 +23,7 @@ namespace shmemg {
 
 enum XKind { X_COPY = 0, X_A2A = 1, X_BCAST = 2, X_FCOLLECT = 3 };
 constexpr int XFER_THREADS = 512;
-constexpr int XFER_U = 4;
+constexpr int XFER_U = 4;  // vectors in flight per thread
 constexpr int RED_THREADS = 256;
 constexpr int RED_U = 2;
 
@@ -34,12 +35,17 @@ struct Xfer {
     int root;
     int dst_pe, src_pe;                // X_COPY
     uint64_t dst_off, src_off;
-    uint64_t seg_vec;                  // vectors per segment
-    uint64_t chunk_vec;                // vectors per item
+    uint64_t segb;                     // bytes per segment
+    uint64_t chunk_vec;                // 16-byte vectors per item
     uint64_t chunks_per_seg;
     uint64_t nitems;                   // items per group
     int mgroups;                       // broadcast / fcollect: destination members split over this many items
+    uint32_t gshift;                   // log2 of the threads that share an item
 };
+
+__device__ __forceinline__ uint64_t xdiv(uint64_t a, uint64_t b) {  // (32-bit where both fit: a fraction of the 64-bit cost)
+    return ((a | b) >> 32) == 0 ? (uint64_t)((uint32_t)a / (uint32_t)b) : a / b;
+}
 
 // Item -> (segment, chunk, member group); a replicating item stores to members
 // [mg*size/mgroups, (mg+1)*size/mgroups) of the team.
@@ -49,70 +55,183 @@ struct XItem {
 };
 __device__ __forceinline__ XItem xitem(const Xfer &x, uint64_t item) {
     XItem t;
-    const uint64_t mg = item % (uint64_t)x.mgroups, rest = item / (uint64_t)x.mgroups;
-    t.seg = rest / x.chunks_per_seg;
+    const uint64_t rest = x.mgroups > 1 ? xdiv(item, (uint64_t)x.mgroups) : item, mg = item - rest * (uint64_t)x.mgroups;
+    t.seg = x.chunks_per_seg > 1 ? xdiv(rest, x.chunks_per_seg) : rest;
     t.ch = rest - t.seg * x.chunks_per_seg;
     t.r0 = (int)(mg * (uint64_t)x.size / (uint64_t)x.mgroups);
     t.r1 = (int)((mg + 1) * (uint64_t)x.size / (uint64_t)x.mgroups);
     return t;
 }
 
-template <typename V>
-__device__ __forceinline__ void xfer_items(const Xfer &x, uint64_t first, uint64_t step) {
-    const int grp = blockIdx.y;
-    const int base_pe = x.start + grp * x.gstride;
-    for (uint64_t item = first; item < x.nitems; item += step) {
-        const XItem it = xitem(x, item);
-        const uint64_t seg = it.seg, ch = it.ch;
-        uint64_t v0 = ch * x.chunk_vec;
-        uint64_t nv = x.seg_vec - v0 < x.chunk_vec ? x.seg_vec - v0 : x.chunk_vec;
-        const uint64_t segb = x.seg_vec * sizeof(V);
-        const V *src;
-        V *dst = nullptr;
-        uint64_t dst_off = x.dst_off;
-        bool replicate = false;
-        if (x.kind == X_COPY) {
-            src = (const V *)(x.heap + (uint64_t)x.src_pe * x.H + x.src_off);
-            dst = (V *)(x.heap + (uint64_t)x.dst_pe * x.H + x.dst_off);
-        } else if (x.kind == X_A2A) {
-            int i = (int)(seg / (uint64_t)x.size), j = (int)(seg - (uint64_t)i * x.size);
-            src = (const V *)(x.heap + (uint64_t)(base_pe + i * x.stride) * x.H + x.src_off + (uint64_t)j * segb);
-            dst = (V *)(x.heap + (uint64_t)(base_pe + j * x.stride) * x.H + x.dst_off + (uint64_t)i * segb);
-        } else if (x.kind == X_BCAST) {
-            src = (const V *)(x.heap + (uint64_t)(base_pe + x.root * x.stride) * x.H + x.src_off);
-            replicate = true;
-        } else {  // X_FCOLLECT: source = member seg, placed at block seg of every dst
-            src = (const V *)(x.heap + (uint64_t)(base_pe + (int)seg * x.stride) * x.H + x.src_off);
-            dst_off = x.dst_off + seg * segb;
-            replicate = true;
+// the 16 bytes that start m bytes into a (0 < m < 16) and run on into b
+__device__ __forceinline__ uint4 xshift(const uint4 &a, const uint4 &b, uint32_t m) {
+    const uint32_t r = (m & 3) * 8;
+    uint32_t w0, w1, w2, w3, w4;
+    switch (m >> 2) {
+    case 0: w0 = a.x, w1 = a.y, w2 = a.z, w3 = a.w, w4 = b.x; break;
+    case 1: w0 = a.y, w1 = a.z, w2 = a.w, w3 = b.x, w4 = b.y; break;
+    case 2: w0 = a.z, w1 = a.w, w2 = b.x, w3 = b.y, w4 = b.z; break;
+    default: w0 = a.w, w1 = b.x, w2 = b.y, w3 = b.z, w4 = b.w; break;
+    }
+    return make_uint4(__funnelshift_r(w0, w1, r), __funnelshift_r(w1, w2, r), __funnelshift_r(w2, w3, r),
+                      __funnelshift_r(w3, w4, r));
+}
+
+// `bytes` (< 16) of a segment's end outside its 16-byte vectors, to nd destinations `step`
+// apart, in the widest units (8 bytes at most) that its addresses and length share (`bits`:
+// all of them or-ed), so that a word stays one store
+__device__ __noinline__ void xedge(uint8_t *d, uint64_t step, int nd, const uint8_t *s, uint32_t bytes, uint64_t bits,
+                                      uint32_t lane, uint32_t gsz) {
+    auto put = [&](auto unit) {
+        using W = decltype(unit);
+        for (uint32_t k = lane; k < bytes / sizeof(W); k += gsz) {
+            const W v = shmemg_ld_cg((const W *)s + k);
+            for (int r = 0; r < nd; r++) ((W *)(d + (uint64_t)r * step))[k] = v;
         }
-        V buf[XFER_U];
+    };
+    if ((bits & 7) == 0) put(uint2());
+    else if ((bits & 3) == 0) put(uint32_t());
+    else if ((bits & 1) == 0) put(uint16_t());
+    else put(uint8_t());
+}
+
+// One item's part of a segment: `nv` vectors from v0 on, stored on the destination's 16-byte
+// boundaries, and the bytes before the first and after the last vector (< 16 each).
+struct XPart {
+    const uint8_t *s;
+    uint8_t *d;
+    uint64_t step;     // replicate: from one member's copy to the next
+    int nd;            // destinations
+    uint32_t head, tail;
+    uint64_t nvec, v0;
+    uint32_t nv;
+    uint64_t bits;     // both addresses and the length, or-ed
+    uint32_t m;        // the source's offset from its 16-byte boundaries, after the head
+    const uint4 *src;  // the aligned vector that holds (the start of) vector v0
+    bool first, last;  // the item with the head, with the tail
+};
+template <bool SHIFT>
+__device__ __forceinline__ XPart xpart(const Xfer &x, uint64_t item, int base_pe) {
+    const XItem it = xitem(x, item);
+    const uint64_t seg = it.seg, segb = x.segb;
+    XPart p;
+    p.step = 0;
+    p.nd = 1;
+    if (x.kind == X_COPY) {
+        p.s = x.heap + (uint64_t)x.src_pe * x.H + x.src_off;
+        p.d = x.heap + (uint64_t)x.dst_pe * x.H + x.dst_off;
+    } else if (x.kind == X_A2A) {
+        const int i = (int)xdiv(seg, (uint64_t)x.size), j = (int)(seg - (uint64_t)i * x.size);
+        p.s = x.heap + (uint64_t)(base_pe + i * x.stride) * x.H + x.src_off + (uint64_t)j * segb;
+        p.d = x.heap + (uint64_t)(base_pe + j * x.stride) * x.H + x.dst_off + (uint64_t)i * segb;
+    } else {  // broadcast: the root's source; fcollect: member seg's, placed at block seg of every dst
+        const int from = x.kind == X_BCAST ? x.root : (int)seg;
+        p.s = x.heap + (uint64_t)(base_pe + from * x.stride) * x.H + x.src_off;
+        p.d = x.heap + (uint64_t)(base_pe + it.r0 * x.stride) * x.H + x.dst_off + (x.kind == X_BCAST ? 0 : seg * segb);
+        p.step = (uint64_t)x.stride * x.H;
+        p.nd = it.r1 - it.r0;
+    }
+    p.bits = (uint64_t)p.s | (uint64_t)p.d | segb;
+    const uint32_t to_line = (uint32_t)(-(intptr_t)p.d) & 15u;
+    p.head = !SHIFT ? 0 : to_line < segb ? to_line : (uint32_t)segb;
+    p.nvec = (segb - p.head) / 16;
+    p.tail = !SHIFT ? 0 : (uint32_t)(segb - p.head) & 15u;
+    p.v0 = it.ch * x.chunk_vec;
+    p.nv = p.v0 >= p.nvec ? 0u : (uint32_t)(p.nvec - p.v0 < x.chunk_vec ? p.nvec - p.v0 : x.chunk_vec);
+    p.m = !SHIFT ? 0 : (uint32_t)(uintptr_t)(p.s + p.head) & 15u;
+    p.src = (const uint4 *)(p.s + p.head - p.m) + p.v0;
+    p.first = it.ch == 0;
+    p.last = it.ch == x.chunks_per_seg - 1;
+    return p;
+}
+__device__ __forceinline__ void xedges(const XPart &p, uint32_t lane, uint32_t gsz) {
+    if (p.head && p.first) xedge(p.d, p.step, p.nd, p.s, p.head, p.bits, lane, gsz);
+    if (p.tail && p.last) {
+        const uint64_t at = p.head + p.nvec * 16;
+        xedge(p.d + at, p.step, p.nd, p.s + at, p.tail, p.bits, lane, gsz);
+    }
+}
+// U vectors of a part, i0 + u * gsz, loaded before any is used.  Where the source lies off its boundaries (SHIFT), a
+// vector is put together from the two aligned ones it spans (the second is an L1 hit: the
+// neighbouring thread's first).  Both hold bytes of the segment, and partitions are
+// 256-byte multiples, so no load leaves a partition.
+template <bool SHIFT, int U>
+__device__ __forceinline__ void xload(const XPart &p, uint32_t i0, uint32_t gsz, uint4 (&buf)[U]) {
+    if (!SHIFT || p.m == 0) {
 #pragma unroll
-        for (int u = 0; u < XFER_U; u++) {
-            uint64_t idx = threadIdx.x + (uint64_t)u * blockDim.x;
-            if (idx < nv) buf[u] = shmemg_ld_cg(src + v0 + idx);
-        }
-        if (!replicate) {
+        for (int u = 0; u < U; u++)
+            if (i0 + u * gsz < p.nv) buf[u] = __ldcg(p.src + i0 + u * gsz);
+    } else {
+        uint4 nx[U];
 #pragma unroll
-            for (int u = 0; u < XFER_U; u++) {
-                uint64_t idx = threadIdx.x + (uint64_t)u * blockDim.x;
-                if (idx < nv) dst[v0 + idx] = buf[u];
+        for (int u = 0; u < U; u++)
+            if (i0 + u * gsz < p.nv) {
+                buf[u] = __ldca(p.src + i0 + u * gsz);
+                nx[u] = __ldca(p.src + i0 + u * gsz + 1);
             }
-        } else {
-            for (int r = it.r0; r < it.r1; r++) {
-                V *d = (V *)(x.heap + (uint64_t)(base_pe + r * x.stride) * x.H + dst_off);
 #pragma unroll
-                for (int u = 0; u < XFER_U; u++) {
-                    uint64_t idx = threadIdx.x + (uint64_t)u * blockDim.x;
-                    if (idx < nv) d[v0 + idx] = buf[u];
-                }
-            }
-        }
+        for (int u = 0; u < U; u++) buf[u] = xshift(buf[u], nx[u], p.m);
     }
 }
 
-template <typename V>
-__global__ void __launch_bounds__(XFER_THREADS) k_xfer(Xfer x) { xfer_items<V>(x, blockIdx.x, gridDim.x); }
+template <bool SHIFT, bool REP>
+__device__ __forceinline__ void xfer_items(const Xfer &x) {
+    const int base_pe = x.start + blockIdx.y * x.gstride;
+    const uint32_t gsz = 1u << x.gshift, lane = threadIdx.x & (gsz - 1), per = blockDim.x >> x.gshift;
+    for (uint64_t item = (uint64_t)blockIdx.x * per + (threadIdx.x >> x.gshift); item < x.nitems; item += (uint64_t)gridDim.x * per) {
+        const XPart p = xpart<SHIFT>(x, item, base_pe);  // (at most XFER_U vectors a thread)
+        uint4 buf[XFER_U];
+        xload<SHIFT, XFER_U>(p, lane, gsz, buf);
+        uint4 *q = (uint4 *)(p.d + p.head) + p.v0 + lane;
+        for (int r = 0; r < (REP ? p.nd : 1); r++) {
+#pragma unroll
+            for (int u = 0; u < XFER_U; u++)
+                if (lane + u * gsz < p.nv) q[u * gsz] = buf[u];
+            if (REP) q = (uint4 *)((uint8_t *)q + p.step);
+        }
+        if (SHIFT) xedges(p, lane, gsz);
+    }
+}
+
+// SHIFT: segments off the 16-byte boundaries; REP: stored to every team member
+template <bool SHIFT, bool REP>
+__global__ void __launch_bounds__(XFER_THREADS, 2) k_xfer(Xfer x) { xfer_items<SHIFT, REP>(x); }
+
+// Broadcast / fcollect whose blocks lie off the 16-byte boundaries: a CTA puts a chunk of some
+// KiB together in shared memory and thread 0 bulk-stores it to every member -- one TMA store
+// per member where each thread stored each vector to each of them.  Bound by the members'
+// writes: fcollect of 48 x 349524 bytes (822 MB) 274 us with 4-byte copies, 165 with 16-byte
+// vector stores, 123 this way; one chunk per CTA (10 us less than resident CTAs that
+// take chunks in turn).  The shared memory asked for is three times what is used: with the
+// 16 KiB in use alone the same launch took 138 us, at the same CTAs per SM and chunks (the
+// cause is not understood).
+constexpr uint32_t XS_SMEM = 3 * XFER_THREADS * XFER_U * 16;
+__global__ void __launch_bounds__(XFER_THREADS, 2) k_xfer_stage(Xfer x) {
+    extern __shared__ __align__(128) uint4 xs_stage[];
+    const int base_pe = x.start + blockIdx.y * x.gstride;
+    for (uint64_t item = blockIdx.x; item < x.nitems; item += gridDim.x) {
+        const XPart p = xpart<true>(x, item, base_pe);
+        uint4 buf[XFER_U];
+        xload<true, XFER_U>(p, threadIdx.x, XFER_THREADS, buf);
+        if (threadIdx.x == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+        __syncthreads();  // an earlier chunk's stores have read the stage
+#pragma unroll
+        for (int u = 0; u < XFER_U; u++)
+            if (threadIdx.x + u * XFER_THREADS < p.nv) xs_stage[threadIdx.x + u * XFER_THREADS] = buf[u];
+        xedges(p, threadIdx.x, XFER_THREADS);
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the stage's generic writes -> bulk copy engine
+        __syncthreads();
+        if (threadIdx.x == 0 && p.nv) {
+            uint8_t *q = p.d + p.head + 16 * p.v0;
+            for (int r = 0; r < p.nd; r++, q += p.step)
+                asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(q),
+                             "r"(shmemg_smem_u32(xs_stage)), "r"(16 * p.nv)
+                             : "memory");
+            asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+        }
+    }
+    if (threadIdx.x == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+}
 
 // ------------------------------------------------------------------ bulk (TMA) variant
 // One thread per CTA streams the CTA's items (chunks of XB_CHUNK bytes) through an
@@ -137,7 +256,7 @@ __device__ __forceinline__ XChunk xchunk(const Xfer &x, uint64_t item, int base_
     const uint64_t seg = it.seg, ch = it.ch;
     c.r0 = it.r0;
     c.r1 = it.r1;
-    const uint64_t segb = x.seg_vec, off = ch * XB_CHUNK;
+    const uint64_t segb = x.segb & ~(uint64_t)15, off = ch * XB_CHUNK;
     c.bytes = (uint32_t)(segb - off < XB_CHUNK ? segb - off : XB_CHUNK);
     c.replicate = false;
     c.dst = nullptr;
@@ -164,8 +283,20 @@ __device__ __forceinline__ XChunk xchunk(const Xfer &x, uint64_t item, int base_
 __global__ void __launch_bounds__(32) k_xfer_bulk(Xfer x, uint8_t *state, uint64_t timeout_ns) {
     extern __shared__ __align__(128) uint8_t ring[];
     __shared__ __align__(8) uint64_t bars[XB_STAGES];
-    if (threadIdx.x != 0) return;
     const int base_pe = x.start + blockIdx.y * x.gstride;
+    if (threadIdx.x != 0) {
+        // the other lanes of the first CTAs: the bytes past the last 16-byte multiple (copy, broadcast)
+        const uint32_t tail = (uint32_t)(x.segb & 15);
+        if (tail && blockIdx.x < (uint32_t)x.mgroups) {
+            const uint64_t at = x.segb - tail;
+            const int from = x.kind == X_COPY ? x.src_pe : base_pe + x.root * x.stride;
+            const int r0 = (int)((uint64_t)blockIdx.x * x.size / x.mgroups), r1 = (int)((uint64_t)(blockIdx.x + 1) * x.size / x.mgroups);
+            const int to = x.kind == X_COPY ? x.dst_pe : base_pe + r0 * x.stride;
+            xedge(x.heap + (uint64_t)to * x.H + x.dst_off + at, (uint64_t)x.stride * x.H, x.kind == X_COPY ? 1 : r1 - r0,
+                  x.heap + (uint64_t)from * x.H + x.src_off + at, tail, x.segb, threadIdx.x - 1, 31);
+        }
+        return;
+    }
     if (x.nitems <= blockIdx.x) return;
     const uint64_t count = (x.nitems - blockIdx.x + gridDim.x - 1) / gridDim.x;
     for (int s = 0; s < XB_STAGES; s++)
@@ -211,20 +342,20 @@ __global__ void __launch_bounds__(32) k_xfer_bulk(Xfer x, uint8_t *state, uint64
     asm volatile("fence.proxy.async.global;" ::: "memory");
 }
 
-// put-with-signal: the copy, then the last CTA to finish releases the signal
-template <typename V>
-__global__ void __launch_bounds__(XFER_THREADS) k_put_signal(Xfer x, uint64_t *sig, uint64_t val, int op,
-                                                             uint32_t *done) {
-    xfer_items<V>(x, blockIdx.x, gridDim.x);
+// put-with-signal: the copy, then the last CTA to finish releases the signal (one CTA needs
+// no count: the signal's release covers its threads' stores, ordered before it by the barrier)
+template <bool SHIFT>
+__global__ void __launch_bounds__(XFER_THREADS, 2) k_put_signal(Xfer x, uint64_t *sig, uint64_t val, int op, uint32_t *done) {
+    xfer_items<SHIFT, false>(x);
     __syncthreads();
     if (threadIdx.x == 0) {
-        shmemg_d_fence_gpu();
-        uint32_t d = atomicAdd(done, 1u);
-        if (d == gridDim.x - 1) {
+        if (gridDim.x > 1) {
+            shmemg_d_fence_gpu();
+            if (atomicAdd(done, 1u) != gridDim.x - 1) return;
             *done = 0;
             shmemg_d_fence_gpu();
-            shmemg_d_signal_op(sig, val, op);
         }
+        shmemg_d_signal_op(sig, val, op);
     }
 }
 
@@ -438,10 +569,6 @@ __global__ void k_wait(shmemg_device_ctx_t c, const uint64_t *sig, int cmp, uint
 }
 
 // ------------------------------------------------------------------ launch helpers
-static int vec_width(uint64_t m) {
-    return (m & 15) == 0 ? 16 : (m & 7) == 0 ? 8 : (m & 3) == 0 ? 4 : (m & 1) == 0 ? 2 : 1;
-}
-
 // Destination members per item of a replicating transfer (broadcast, fcollect): a
 // launch with fewer segment chunks than resident CTAs splits each chunk's member stores
 // over several items (each reads the chunk -- from L2 after the first), so the stores
@@ -450,27 +577,84 @@ static int member_groups(const Xfer &x, uint64_t items, uint64_t cap, int ngroup
     if ((x.kind != X_BCAST && x.kind != X_FCOLLECT) || items == 0) return 1;
     if (ngroups > 1) cap = cap / (uint64_t)ngroups > 0 ? cap / (uint64_t)ngroups : 1;
     if (items >= cap) return 1;
-    const uint64_t g = (cap + items - 1) / items;
+    const uint64_t g = cap / items;
     return (int)(g < (uint64_t)x.size ? g : (uint64_t)x.size);
 }
 
-template <typename V>
-static int launch_xfer_v(Xfer x, int ngroups, cudaStream_t s, uint64_t *sig, uint64_t val, int op, uint32_t *done) {
-    x.seg_vec /= sizeof(V);
-    x.chunk_vec = (uint64_t)XFER_THREADS * XFER_U;
-    x.chunks_per_seg = (x.seg_vec + x.chunk_vec - 1) / x.chunk_vec;
-    if (x.chunks_per_seg == 0) x.chunks_per_seg = 1;
-    uint64_t nseg = x.kind == X_A2A ? (uint64_t)x.size * x.size : x.kind == X_FCOLLECT ? (uint64_t)x.size : 1;
-    x.nitems = x.seg_vec ? nseg * x.chunks_per_seg : 0;
-    if (x.nitems == 0 && !sig) return SHMEMG_SUCCESS;
-    const void *kfn = sig ? (const void *)k_put_signal<V> : (const void *)k_xfer<V>;
-    const uint64_t cap = (uint64_t)ctas_for(kfn, XFER_THREADS, 0);
+static uint64_t xfer_segments(const Xfer &x) {
+    return x.kind == X_A2A ? (uint64_t)x.size * x.size : x.kind == X_FCOLLECT ? (uint64_t)x.size : 1;
+}
+
+// the dynamic shared memory granted to kernel `k` (once per kernel)
+static bool smem_ready(const void *k, uint32_t bytes) {
+    static std::mutex mu;
+    static std::unordered_map<const void *, bool> ok;
+    std::lock_guard<std::mutex> lk(mu);
+    auto it = ok.find(k);
+    if (it != ok.end()) return it->second;
+    const bool g = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess;
+    if (!g) cudaGetLastError();
+    ok[k] = g;
+    return g;
+}
+
+// Broadcast / fcollect off the boundaries with blocks of XS_MIN bytes or more: k_xfer_stage (a
+// bulk copy below a few KiB costs the copy engine as much as one of 4 KiB).
+constexpr uint64_t XS_MIN = 4u << 10;
+static int launch_xfer_stage(Xfer x, int ngroups, cudaStream_t s) {
+    const uint64_t nseg = xfer_segments(x), vecs = x.segb / 16;
+    const uint64_t cap = (uint64_t)ctas_for((const void *)k_xfer_stage, XFER_THREADS, XS_SMEM);
+    // chunks of 8 KiB, or of up to 16 where that is more than the resident CTAs take at once
+    // (32 KiB ones leave a last wave half empty: 148 us against 126), equal within a block
+    const uint64_t most = nseg * ((vecs + XFER_THREADS - 1) / XFER_THREADS) > cap ? 2 * XFER_THREADS : XFER_THREADS;
+    x.chunks_per_seg = (vecs + most - 1) / most;
+    x.chunk_vec = (vecs + x.chunks_per_seg - 1) / x.chunks_per_seg;
+    x.nitems = nseg * x.chunks_per_seg;
     x.mgroups = member_groups(x, x.nitems, cap, ngroups);
     x.nitems *= (uint64_t)x.mgroups;
-    const uint64_t gx = balanced_grid(x.nitems, cap, ngroups);
+    dim3 grid((unsigned)(x.nitems < (1u << 30) ? x.nitems : 1u << 30), (unsigned)ngroups);
+    k_xfer_stage<<<grid, XFER_THREADS, XS_SMEM, s>>>(x);
+    return cuda_rc(cudaGetLastError());
+}
+
+// Threads per item: enough that a segment's vectors go one to a thread, a whole CTA at most
+// (segments of a few vectors share a CTA); fewer, with up to U vectors each, once the
+// segments fill the resident CTAs.  Vectors per item: as few per thread as keep the items
+// within the resident CTAs, so a middle-sized transfer spreads over the GPU.
+template <bool SHIFT>
+static int launch_xfer_vec(Xfer x, int ngroups, cudaStream_t s, uint64_t *sig, uint64_t val, int op, uint32_t *done) {
+    constexpr uint64_t U = XFER_U;
+    const uint64_t nseg = xfer_segments(x), vecs = x.segb >= 16 ? x.segb / 16 : 1;
+    const bool rep = x.kind == X_BCAST || x.kind == X_FCOLLECT;
+    const void *kfn = sig ? (const void *)k_put_signal<SHIFT> : rep ? (const void *)k_xfer<SHIFT, true> : (const void *)k_xfer<SHIFT, false>;
+    const uint64_t cap = (uint64_t)ctas_for(kfn, XFER_THREADS, 0);
+    const uint64_t threads = cap * XFER_THREADS / (uint64_t)ngroups + 1;
+    uint32_t g = 3;
+    while ((1u << g) < XFER_THREADS && (1ull << g) < vecs) g++;
+    while (g > 3 && nseg << g > threads && U << (g - 1) >= vecs) g--;
+    x.gshift = g;
+    uint64_t u = 1;
+    while (u < U && (nseg * ((vecs + (u << g) - 1) / (u << g))) << g > threads) u++;
+    x.chunk_vec = u << g;
+    x.chunks_per_seg = (vecs + x.chunk_vec - 1) / x.chunk_vec;
+    x.nitems = x.segb ? nseg * x.chunks_per_seg : 0;
+    if (x.nitems == 0 && !sig) return SHMEMG_SUCCESS;
+    x.mgroups = member_groups(x, x.nitems, (cap * XFER_THREADS) >> g, ngroups);
+    x.nitems *= (uint64_t)x.mgroups;
+    // CTAs of XFER_THREADS, or as many threads as a small transfer has work for
+    unsigned block = XFER_THREADS;
+    while (block > 32 && (uint64_t)(block / 2) >= x.nitems << g) block /= 2;
+    const uint64_t per = block >> g;
+    // aligned copies take one round of items per CTA and leave the queue to the hardware: a CTA
+    // that waits for nothing but its stores makes room for the next one's loads (alltoall of 64
+    // PEs x 64 KiB per pair 85.9 -> 83.0 us, 24 x 1 MiB 190 -> 179, 0.99 of the copy rate); the
+    // others keep resident CTAs (64 PEs x 60004 B per pair 99.6 us against 106.6)
+    const uint64_t rounds = (x.nitems + per - 1) / per;
+    const uint64_t gx = SHIFT || rep || sig ? balanced_grid(rounds, cap, ngroups) : rounds < (1u << 30) ? rounds : 1u << 30;
     dim3 grid((unsigned)gx, (unsigned)ngroups);
-    if (sig) k_put_signal<V><<<grid, XFER_THREADS, 0, s>>>(x, sig, val, op, done);
-    else k_xfer<V><<<grid, XFER_THREADS, 0, s>>>(x);
+    if (sig) k_put_signal<SHIFT><<<grid, block, 0, s>>>(x, sig, val, op, done);
+    else if (rep) k_xfer<SHIFT, true><<<grid, block, 0, s>>>(x);
+    else k_xfer<SHIFT, false><<<grid, block, 0, s>>>(x);
     return cuda_rc(cudaGetLastError());
 }
 
@@ -488,11 +672,11 @@ static bool bulk_enabled() {
     return on == 1;
 }
 
-// segments of >= one chunk with 16-byte aligned addresses and lengths go to the bulk engine
+// segments of >= one chunk at 16-byte aligned addresses go to the bulk engine (an odd length's
+// last bytes beside it; the blocks of an fcollect of odd length are not aligned)
 static int launch_xfer_bulk(Xfer x, int ngroups, cudaStream_t s) {
-    x.chunks_per_seg = (x.seg_vec + XB_CHUNK - 1) / XB_CHUNK;
-    const uint64_t nseg = x.kind == X_A2A ? (uint64_t)x.size * x.size : x.kind == X_FCOLLECT ? (uint64_t)x.size : 1;
-    x.nitems = nseg * x.chunks_per_seg;
+    x.chunks_per_seg = ((x.segb & ~(uint64_t)15) + XB_CHUNK - 1) / XB_CHUNK;
+    x.nitems = xfer_segments(x) * x.chunks_per_seg;
     const uint64_t cap = (uint64_t)ctas_for((const void *)k_xfer_bulk, 32, XB_SMEM);
     x.mgroups = member_groups(x, x.nitems, cap, ngroups);
     x.nitems *= (uint64_t)x.mgroups;
@@ -501,19 +685,17 @@ static int launch_xfer_bulk(Xfer x, int ngroups, cudaStream_t s) {
     return cuda_rc(cudaGetLastError());
 }
 
-// x.seg_vec carries the segment length in BYTES on entry
 static int launch_xfer(Xfer x, int ngroups, uint64_t align_bits, cudaStream_t s, uint64_t *sig = nullptr,
                        uint64_t val = 0, int op = 0, uint32_t *done = nullptr) {
     // (alltoall's many smaller segments measured faster on the vector path)
-    if (!sig && x.kind != X_A2A && ((align_bits | x.seg_vec) & 15) == 0 && x.seg_vec >= XB_CHUNK && bulk_enabled())
+    if (x.kind == X_FCOLLECT) align_bits |= x.segb;
+    if (!sig && x.kind != X_A2A && (align_bits & 15) == 0 && x.segb >= XB_CHUNK && bulk_enabled())
         return launch_xfer_bulk(x, ngroups, s);
-    switch (vec_width(align_bits | x.seg_vec)) {
-    case 16: return launch_xfer_v<uint4>(x, ngroups, s, sig, val, op, done);
-    case 8: return launch_xfer_v<uint2>(x, ngroups, s, sig, val, op, done);
-    case 4: return launch_xfer_v<uint32_t>(x, ngroups, s, sig, val, op, done);
-    case 2: return launch_xfer_v<uint16_t>(x, ngroups, s, sig, val, op, done);
-    default: return launch_xfer_v<uint8_t>(x, ngroups, s, sig, val, op, done);
-    }
+    if (((align_bits | x.segb) & 15) == 0) return launch_xfer_vec<false>(x, ngroups, s, sig, val, op, done);
+    if ((x.kind == X_BCAST || x.kind == X_FCOLLECT) && x.size > 1 && x.segb >= XS_MIN && bulk_enabled() &&
+        smem_ready((const void *)k_xfer_stage, XS_SMEM))
+        return launch_xfer_stage(x, ngroups, s);
+    return launch_xfer_vec<true>(x, ngroups, s, sig, val, op, done);
 }
 
 static Xfer xfer_base() {
@@ -539,7 +721,7 @@ static int rma(void *dst, const void *src, uint64_t n, int dst_pe, int src_pe, v
     x.src_pe = src_pe;
     x.dst_off = doff;
     x.src_off = soff;
-    x.seg_vec = n;
+    x.segb = n;
     return launch_xfer(x, 1, doff | soff, to_stream(stream));
 }
 
@@ -562,19 +744,6 @@ static bool rb_shape(int P, uint32_t *chunk, uint32_t *stages) {
     return P >= 48 && P <= 64;
 }
 
-// the ring's shared memory granted to kernel `k` (once per instantiation)
-static bool red_bulk_ready(const void *k) {
-    static std::mutex mu;
-    static std::unordered_map<const void *, bool> ok;
-    std::lock_guard<std::mutex> lk(mu);
-    auto it = ok.find(k);
-    if (it != ok.end()) return it->second;
-    const bool g = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, RB_SMEM) == cudaSuccess;
-    if (!g) cudaGetLastError();
-    ok[k] = g;
-    return g;
-}
-
 template <typename V, typename T, int OP>
 static int launch_red_v(Red r, int ngroups, cudaStream_t s) {
     r.nvec /= (sizeof(V) / sizeof(T));
@@ -585,7 +754,7 @@ static int launch_red_v(Red r, int ngroups, cudaStream_t s) {
         // integer teams of 48..64 members with 128 KiB .. 16 MiB per member: the bulk ring
         // (above 16 MiB both forms run at the HBM rate and the register form is the steadier)
         if ((r.H & 15) == 0 && r.nvec * sizeof(V) >= red_bulk_min() && r.nvec * sizeof(V) <= RB_MAX_BYTES &&
-            rb_shape(r.size, &r.rb_chunk, &r.rb_stages) && red_bulk_ready((const void *)k_reduce_bulk<T, V, OP>)) {
+            rb_shape(r.size, &r.rb_chunk, &r.rb_stages) && smem_ready((const void *)k_reduce_bulk<T, V, OP>, RB_SMEM)) {
             const uint64_t C = r.rb_chunk, nchunks = (r.nvec * sizeof(V) + C - 1) / C;
             const uint64_t cap = (uint64_t)ctas_for((const void *)k_reduce_bulk<T, V, OP>, RB_THREADS, RB_SMEM);
             dim3 grid((unsigned)balanced_grid(nchunks, cap, ngroups), (unsigned)ngroups);
@@ -700,7 +869,7 @@ int shmemg_putmem_signal(void *dst, const void *src, uint64_t n, uint64_t *sig, 
     x.src_pe = issuer;
     x.dst_off = doff;
     x.src_off = soff;
-    x.seg_vec = n;
+    x.segb = n;
     uint32_t *done = (uint32_t *)(S.base + SHMEMG_SCRATCH_OFF + SCR_SIGNAL_DONE) +
                      (S.call_seq++ % SCR_SIGNAL_DONE_SLOTS);
     uint64_t *sig_addr = (uint64_t *)(S.heap + (uint64_t)pe * S.H + goff);
@@ -745,7 +914,7 @@ int shmemg_broadcastmem(shmemg_team_t team, void *dst, const void *src, uint64_t
     x.root = root;
     x.dst_off = doff;
     x.src_off = soff;
-    x.seg_vec = n;
+    x.segb = n;
     return launch_xfer(x, t.ngroups, doff | soff, to_stream(stream));
 }
 
@@ -758,7 +927,7 @@ int shmemg_fcollectmem(shmemg_team_t team, void *dst, const void *src, uint64_t 
     Xfer x = team_xfer(t, X_FCOLLECT);
     x.dst_off = doff;
     x.src_off = soff;
-    x.seg_vec = n;
+    x.segb = n;
     return launch_xfer(x, t.ngroups, doff | soff, to_stream(stream));
 }
 
@@ -772,7 +941,7 @@ int shmemg_alltoallmem(shmemg_team_t team, void *dst, const void *src, uint64_t 
     Xfer x = team_xfer(t, X_A2A);
     x.dst_off = doff;
     x.src_off = soff;
-    x.seg_vec = n;
+    x.segb = n;
     return launch_xfer(x, t.ngroups, doff | soff, to_stream(stream));
 }
 

@@ -7,6 +7,7 @@ import torch
 import workloads as W
 from test_gpu_amo_quant_batch import _check_stream, _table_heap
 from test_gpu_halo import _run as _run_halo
+from gpu_util import download, first_diff, random_heap, upload
 
 pytestmark = pytest.mark.gpu
 
@@ -56,3 +57,57 @@ def test_halo_captured_and_replayed(sg, heapf, orc, nx, ny):
     for p in range(px * py):
         t = want[p // px * ny:(p // px + 1) * ny, p % px * nx:(p % px + 1) * nx]
         assert np.array_equal(h.view(tiles, p, torch.float32, n).cpu().numpy().reshape(ny, nx).view(np.uint32), t.view(np.uint32))
+
+
+RAGGED = [1, 2, 3, 7, 8, 9, 15, 16, 17, 31, 33, 100, 4095, 8191, 8192, 32767, 32768, 32773, 70004, 262147]
+
+
+@pytest.mark.parametrize("ds,ss", [(0, 0), (0, 1), (1, 0), (3, 3), (4, 12), (8, 0), (15, 2), (5, 14)])
+def test_rma_any_alignment(sg, heapf, ds, ss):
+    """Heads, bodies and tails of put, get and put_signal: no byte outside the range changes."""
+    npes, H = 3, 1 << 20
+    h = heapf(npes, H)
+    for k, n in enumerate(RAGGED):
+        want = random_heap(npes, H, 100 + k)
+        upload(h, want)
+        m = want.reshape(npes, H)
+        dst, src = 300000 + ds, 4096 + ss   # (300000 is a multiple of 32: the shift alone decides)
+        sg.putmem(h.base + dst, h.base + src, n, 2, 0)
+        m[2, dst:dst + n] = m[0, src:src + n]
+        sg.getmem(h.base + dst, h.base + src, n, 2, 1)
+        m[1, dst:dst + n] = m[2, src:src + n]
+        sg.putmem_signal(h.base + dst + 300032, h.base + src, n, h.base + 8, 3, sg.SIGNAL_SET, 0, 1)
+        m[0, dst + 300032:dst + 300032 + n] = m[1, src:src + n]
+        m[0, 8:16].view(np.uint64)[0] = 3
+        assert first_diff(download(h), want) is None, n
+
+
+@pytest.mark.parametrize("P,start,stride", [(1, 4, 1), (3, 1, 2), (16, 0, 1)])
+@pytest.mark.parametrize("ds,ss", [(0, 0), (4, 0), (7, 13)])
+def test_collectives_of_ragged_blocks(sg, heapf, P, start, stride, ds, ss):
+    npes, H = 16, 1 << 20
+    h = heapf(npes, H)
+    team = sg.team_split_strided(sg.TEAM_WORLD, start, stride, P)
+    pes = [start + r * stride for r in range(P)]
+    dst, src = 524288 + ds, 1024 + ss
+    for k, n in enumerate([1, 3, 4, 20, 130, 4092, 4100, 8195, 20004] + ([32780, 100003] if P < 4 else [])):
+        for op in ("broadcast", "fcollect", "alltoall"):
+            want = random_heap(npes, H, 7 * k + len(op))
+            upload(h, want)
+            m = want.reshape(npes, H)
+            old = m.copy()
+            if op == "broadcast":
+                sg.broadcastmem(team, h.base + dst, h.base + src, n, P - 1)
+            elif op == "fcollect":
+                sg.fcollectmem(team, h.base + dst, h.base + src, n)
+            else:
+                sg.alltoallmem(team, h.base + dst, h.base + src, n)
+            for j, q in enumerate(pes):
+                if op == "broadcast":
+                    m[q, dst:dst + n] = old[pes[-1], src:src + n]
+                    continue
+                for i, p in enumerate(pes):
+                    s = src if op == "fcollect" else src + j * n
+                    m[q, dst + i * n:dst + (i + 1) * n] = old[p, s:s + n]
+            assert first_diff(download(h), want) is None, (op, n)
+    sg.team_destroy(team)
