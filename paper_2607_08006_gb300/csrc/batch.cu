@@ -2,8 +2,8 @@
 // captured in a CUDA graph (a batching extension of the team reductions the paper
 // inherits from OpenSHMEM 1.6, Sec. 6.3).
 //
-// Work items are (team, tile) pairs planned on the host, largest team first (cost =
-// members x elements x bytes); CTAs of a persistent grid take items from a device
+// Work items are (team, tile) pairs planned on the host, costliest first (members x
+// elements x bytes); CTAs of a persistent grid take items from a device
 // counter.  Each item is a slice-owner reduction of one tile over the team's members:
 // fp32 by the fixed rank-pairwise tree, int64 exactly, bf16/e4m3 payloads dequantised
 // and accumulated with Neumaier's compensated sum.  The last CTA to leave resets the
@@ -23,6 +23,7 @@ namespace shmemg {
 
 constexpr int B_THREADS = 256;
 constexpr int B_DEEP_QM = 16;
+constexpr int B_SMALL_QM = 16;  // members ahead where a thread has four elements
 // Two kernels (the plan's `deep` picks one): the lean one holds 85 registers for 3 CTAs per
 // SM, with 16 members' loads in flight in the fp32 tree and 8 quantised members loaded
 // ahead; the deep one holds 128 registers for 2 CTAs per SM and loads further ahead.
@@ -34,6 +35,7 @@ enum BKind { BK_F32 = 0, BK_I64 = 1, BK_BF16 = 2, BK_E4M3 = 3 };
 struct BTeam {
     int32_t start, size, kind, vec;
     uint64_t n, d_off, s_off, sc_off;
+    uint64_t tile;        // elements per work item
 };
 
 struct BArgs {
@@ -42,47 +44,55 @@ struct BArgs {
     const BTeam *teams;
     const uint2 *items;   // (team, tile)
     uint32_t nitems;
-    uint32_t tile;        // elements per item
     uint32_t *counter;    // [0] next item, [1] CTAs done
 };
 
 // quantised tile: full chunks of blockDim x E elements accumulate into shared memory (two
 // buffers, alternated across the CTA's chunks) and are bulk-stored to every member (bit 1
-// of t.vec: 16-byte aligned codes and outputs); the rest runs E (or 4) elements per thread
+// of t.vec: 16-byte aligned codes and outputs), then chunks of blockDim x 4, the smallest
+// item of the per-team plan; the rest runs 4 elements per thread
 template <int FMT, int M>
 __device__ __forceinline__ void batch_qsum(const BArgs &a, const BTeam &t, uint64_t e0, uint64_t e1, float (*s_out)[B_THREADS * 16],
                                            int &buf) {
-    constexpr int E = QWide<FMT>::E;
-    const uint64_t CH = (uint64_t)blockDim.x * E;
+    const uint64_t CH = (uint64_t)blockDim.x * QWide<FMT>::E, SMALL = (uint64_t)blockDim.x * 4;
     uint64_t f0 = e0;
     if (t.vec & 2) {
         for (; f0 + CH <= e1; f0 += CH) {
             qsum_chunk_tma<FMT, M>(a.heap, a.H, t.start, 1, t.size, t.d_off, t.s_off, t.sc_off, f0, s_out[buf]);
             buf ^= 1;
         }
-    }
-    for (uint64_t q = f0 / E + threadIdx.x; q * E < e1; q += blockDim.x) {
-        const uint64_t f = q * E;
-        if ((t.vec & 2) && f + E <= e1) {
-            qsum_wide<FMT, M>(a.heap, a.H, t.start, 1, t.size, t.d_off, t.s_off, t.sc_off, f);
-        } else {
-            for (int k = 0; k < E / 4 && f + 4 * k < e1; k++)
-                qsum4<FMT>(a.heap, a.H, t.start, 1, t.size, t.d_off, t.s_off, t.sc_off, f + 4 * k, t.n,
-                           (t.vec & 1) && f + 4 * k + 4 <= t.n);
+        for (; f0 + SMALL <= e1; f0 += SMALL) {
+            qsum_chunk_tma<FMT, B_SMALL_QM, 4>(a.heap, a.H, t.start, 1, t.size, t.d_off, t.s_off, t.sc_off, f0, s_out[buf]);
+            buf ^= 1;
         }
     }
+    for (uint64_t f = f0 + 4 * threadIdx.x; f < e1; f += SMALL)
+        qsum4<FMT, B_SMALL_QM>(a.heap, a.H, t.start, 1, t.size, t.d_off, t.s_off, t.sc_off, f, t.n, (t.vec & 1) != 0);
+}
+
+// exact sums: whole 16-byte vectors where the offsets allow them, the elements past the last one
+// by the threads with the fewest vectors
+template <typename T, typename V, int TREE_MAXB>
+__device__ __forceinline__ void batch_sum(const BArgs &a, const BTeam &t, uint64_t e0, uint64_t e1) {
+    constexpr uint64_t L = sizeof(V) / sizeof(T);
+    uint64_t f = e0;
+    if (((t.d_off | t.s_off | (e0 * sizeof(T))) & 15) == 0) {  // (partitions are 256-byte multiples)
+        shmemg_d_reduce_vecs<T, V, SHMEMG_SUM, TREE_MAXB>({threadIdx.x, blockDim.x}, a.heap, a.H, t.start, 1, t.size, t.d_off,
+                                                          t.s_off, e0 / L, e1 / L);
+        f = e1 / L * L;
+        if (f == e1) return;
+    }
+    shmemg_d_reduce_vecs<T, T, SHMEMG_SUM, TREE_MAXB>({blockDim.x - 1 - threadIdx.x, blockDim.x}, a.heap, a.H, t.start, 1, t.size,
+                                                      t.d_off, t.s_off, f, e1);
 }
 
 template <int MINB>
 __device__ __forceinline__ void batch_item(const BArgs &a, const BTeam &t, uint64_t e0, uint64_t e1, float (*s_out)[B_THREADS * 16],
                                            int &buf) {
-    const shmemg_group g = {threadIdx.x, blockDim.x};
     if (t.kind == BK_F32) {
-        shmemg_d_reduce_elems_t<float, float4, BShape<MINB>::TREE_MAXB>(g, a.heap, a.H, t.start, 1, t.size, t.d_off, t.s_off, e0, e1,
-                                                         SHMEMG_SUM);
+        batch_sum<float, float4, BShape<MINB>::TREE_MAXB>(a, t, e0, e1);
     } else if (t.kind == BK_I64) {
-        shmemg_d_reduce_elems_t<int64_t, longlong2>(g, a.heap, a.H, t.start, 1, t.size, t.d_off, t.s_off, e0, e1,
-                                                    SHMEMG_SUM);
+        batch_sum<int64_t, longlong2, BShape<MINB>::TREE_MAXB>(a, t, e0, e1);
     } else {
         if (t.kind == BK_E4M3) batch_qsum<SHMEMG_FMT_E4M3, BShape<MINB>::QM>(a, t, e0, e1, s_out, buf);
         else batch_qsum<SHMEMG_FMT_BF16, BShape<MINB>::QM>(a, t, e0, e1, s_out, buf);
@@ -102,8 +112,8 @@ __global__ void __launch_bounds__(B_THREADS, MINB) k_batch(BArgs a) {
         if (it >= a.nitems) break;
         const uint2 item = a.items[it];
         const BTeam t = a.teams[item.x];
-        const uint64_t e0 = (uint64_t)item.y * a.tile;
-        const uint64_t e1 = e0 + a.tile < t.n ? e0 + a.tile : t.n;
+        const uint64_t e0 = (uint64_t)item.y * t.tile;
+        const uint64_t e1 = e0 + t.tile < t.n ? e0 + t.tile : t.n;
         batch_item<MINB>(a, t, e0, e1, s_out, buf);
     }
     if (threadIdx.x == 0) {
@@ -125,7 +135,7 @@ using namespace shmemg;
 
 struct shmemg_batch_s {
     std::vector<BTeam> teams;
-    std::vector<uint64_t> cost;
+    std::vector<uint64_t> cost;   // bytes per element of all members
     BTeam *d_teams = nullptr;
     uint2 *d_items = nullptr;
     uint32_t *d_counter = nullptr;
@@ -143,16 +153,44 @@ static void free_graph(shmemg_batch_s *b) {
     b->graph = nullptr;
 }
 
-// (re)plan items for the batch's tile size, upload them and capture the graph
+// Elements per work item of each team.  A given tile size holds for every team.  Without
+// one the items get about equal shares of the bytes, B_SHARES of them per resident CTA, at
+// least what gives every thread one vector (256 x 16 bytes of fp32 and int64, 256 x 4 codes):
+// a uniform tile is too coarse for the largest teams and leaves a few CTAs working on them
+// alone.  64 teams of 2-128 PEs x 256-256 Ki elements (694 MB, 102 us at the copy rate):
+// 514 us with 16384-element tiles (192 items on 456 CTAs), 121 with these; 123 with 8 shares
+// per CTA, 126 with 4 or with half the least sizes.
+constexpr uint64_t B_SHARES = 16;
+static void plan_tiles(shmemg_batch_s *b) {
+    uint64_t total = 0;
+    for (size_t i = 0; i < b->teams.size(); i++) total += b->cost[i] * b->teams[i].n;
+    const uint64_t share = total / ((uint64_t)b->grid * B_SHARES) + 1;
+    for (size_t i = 0; i < b->teams.size(); i++) {
+        BTeam &t = b->teams[i];
+        const uint64_t unit = t.kind == BK_I64 ? 512 : 1024;
+        t.tile = b->tune.tile_elems > 0 ? (uint64_t)b->tune.tile_elems
+                                        : std::min<uint64_t>(std::max<uint64_t>(share / b->cost[i] / unit, 1) * unit, 131072);
+    }
+}
+
+// (re)plan the items, upload them and the teams, and capture the graph
 static int plan_and_capture(shmemg_batch_s *b) {
     State &S = st();
-    const uint32_t tile = (uint32_t)b->tune.tile_elems;
+    int per_sm = 0;
+    const void *kfn = b->tune.deep ? (const void *)k_batch<2> : (const void *)k_batch<3>;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kfn, B_THREADS, 0);
+    if (per_sm < 1) per_sm = 1;
+    int want = b->tune.ctas_per_sm > 0 ? std::min(b->tune.ctas_per_sm, per_sm) : per_sm;
+    b->grid = want * S.sm_count;
+    plan_tiles(b);
+    // costliest items first
     std::vector<int> order(b->teams.size());
     for (size_t i = 0; i < order.size(); i++) order[i] = (int)i;
-    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return b->cost[x] > b->cost[y]; });
+    auto item_cost = [&](int t) { return b->cost[t] * std::min<uint64_t>(b->teams[t].tile, b->teams[t].n); };
+    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return item_cost(x) > item_cost(y); });
     std::vector<uint2> items;
     for (int t : order) {
-        uint64_t tiles = (b->teams[t].n + tile - 1) / tile;
+        uint64_t tiles = (b->teams[t].n + b->teams[t].tile - 1) / b->teams[t].tile;
         for (uint64_t k = 0; k < tiles; k++) items.push_back(make_uint2((unsigned)t, (unsigned)k));
     }
     if (items.size() >= (1ull << 31)) return SHMEMG_ERR_INVALID_ARG;
@@ -163,12 +201,7 @@ static int plan_and_capture(shmemg_batch_s *b) {
     if ((rc = cuda_rc(cudaMemcpy(b->d_items, items.data(), sizeof(uint2) * items.size(), cudaMemcpyHostToDevice))))
         return rc;
     b->nitems = (uint32_t)items.size();
-    int per_sm = 0;
-    const void *kfn = b->tune.deep ? (const void *)k_batch<2> : (const void *)k_batch<3>;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kfn, B_THREADS, 0);
-    if (per_sm < 1) per_sm = 1;
-    int want = b->tune.ctas_per_sm > 0 ? std::min(b->tune.ctas_per_sm, per_sm) : per_sm;
-    b->grid = want * S.sm_count;
+    if ((rc = cuda_rc(cudaMemcpy(b->d_teams, b->teams.data(), sizeof(BTeam) * b->teams.size(), cudaMemcpyHostToDevice)))) return rc;
     if ((uint32_t)b->grid > b->nitems) b->grid = (int)std::max<uint32_t>(b->nitems, 1u);
     free_graph(b);
     cudaStream_t cs;
@@ -179,7 +212,6 @@ static int plan_and_capture(shmemg_batch_s *b) {
     a.teams = b->d_teams;
     a.items = b->d_items;
     a.nitems = b->nitems;
-    a.tile = tile;
     a.counter = b->d_counter;
     rc = cuda_rc(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
     if (!rc) {
@@ -229,15 +261,14 @@ int shmemg_batch_create(const shmemg_coll_desc_t *descs, int count, const shmemg
                     ((t.d_off & 15) == 0 && (t.s_off & 15) == 0 ? 2 : 0);
         }
         b->teams.push_back(t);
-        b->cost.push_back((uint64_t)d.size * d.n * (in_es + out_es));
+        b->cost.push_back((uint64_t)d.size * (in_es + out_es));
     }
-    b->tune.tile_elems = tune && tune->tile_elems > 0 ? tune->tile_elems : 16384;
+    b->tune.tile_elems = tune && tune->tile_elems > 0 ? tune->tile_elems : 0;  // 0: per team
     b->tune.ctas_per_sm = tune ? tune->ctas_per_sm : 0;
     b->tune.threads = B_THREADS;
     b->tune.deep = tune && tune->deep ? 1 : 0;
     if (b->tune.tile_elems % 128) { delete b; return SHMEMG_ERR_INVALID_ARG; }
     int rc = cuda_rc(cudaMalloc(&b->d_teams, sizeof(BTeam) * b->teams.size()));
-    if (!rc) rc = cuda_rc(cudaMemcpy(b->d_teams, b->teams.data(), sizeof(BTeam) * b->teams.size(), cudaMemcpyHostToDevice));
     if (!rc) rc = cuda_rc(cudaMalloc(&b->d_counter, 2 * sizeof(uint32_t)));
     if (!rc) rc = cuda_rc(cudaMemset(b->d_counter, 0, 2 * sizeof(uint32_t)));
     if (!rc) rc = plan_and_capture(b);
@@ -370,6 +401,7 @@ extern "C" int shmemg_batch_reduce_noalloc(const shmemg_coll_desc_t *descs, int 
         t.start = c.start;
         t.size = c.size;
         t.n = c.n;
+        t.tile = tile;
         uint64_t in_es, out_es = 4;
         if (c.dtype == SHMEMG_INT64) { t.kind = BK_I64; in_es = 8; out_es = 8; }
         else if (c.dtype == SHMEMG_FLOAT && c.fmt < 0) { t.kind = BK_F32; in_es = 4; }
@@ -409,7 +441,6 @@ extern "C" int shmemg_batch_reduce_noalloc(const shmemg_coll_desc_t *descs, int 
     a.teams = d->teams;
     a.items = d->items;
     a.nitems = k;
-    a.tile = tile;
     a.counter = d->counter;
     int grid = ctas_for((const void *)k_batch<3>, B_THREADS, 0);
     if ((uint32_t)grid > k) grid = (int)k;

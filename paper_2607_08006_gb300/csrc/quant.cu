@@ -109,7 +109,7 @@ __global__ void __launch_bounds__(Q_THREADS) k_qsum(QSumArgs a) {
     const uint64_t t0 = nfull * CH;
     for (uint64_t f = t0 + 4 * ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x); f < a.n;
          f += 4 * (uint64_t)gridDim.x * blockDim.x)
-        qsum4<FMT>(a.heap, a.H, pe0, a.stride, a.size, a.d_off, a.q_off, a.s_off, f, a.n, a.vec && f + 4 <= a.n);
+        qsum4<FMT>(a.heap, a.H, pe0, a.stride, a.size, a.d_off, a.q_off, a.s_off, f, a.n, a.vec);
 }
 
 }  // namespace shmemg

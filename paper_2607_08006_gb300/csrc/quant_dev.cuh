@@ -90,20 +90,35 @@ struct Neu2 {
     __device__ __forceinline__ uint64_t result() const { return f2_add(sum, c); }
 };
 
-// Elements per thread of the wide path: one 16-byte code load per member.
+// Elements per thread of the widest path: one 16-byte code load per member.
 template <int FMT> struct QWide { static constexpr int E = FMT == SHMEMG_FMT_E4M3 ? 16 : 8; };
 
-// The E dequantised values of one 16-byte code load, as E/2 pairs: decoded exactly to
-// binary32, then one RNE multiply by the block scale each (packed).
-template <int FMT>
-__device__ __forceinline__ void qdecode16(uint4 w, float s, uint64_t *d) {
-    const uint32_t v[4] = {w.x, w.y, w.z, w.w};
+// Words of E codes in memory, and their load (bypassing L1, as every member load).
+template <int FMT, int E> struct QWords { static constexpr int N = E * (FMT == SHMEMG_FMT_E4M3 ? 1 : 2) / 4; };
+template <int N>
+__device__ __forceinline__ void qload(const uint8_t *p, uint32_t (&v)[N]) {
+    static_assert(N == 1 || N == 2 || N == 4, "4, 8 or 16 bytes");
+    if constexpr (N == 4) {
+        const uint4 w = __ldcg((const uint4 *)p);
+        v[0] = w.x, v[1] = w.y, v[2] = w.z, v[3] = w.w;
+    } else if constexpr (N == 2) {
+        const uint2 w = __ldcg((const uint2 *)p);
+        v[0] = w.x, v[1] = w.y;
+    } else {
+        v[0] = __ldcg((const unsigned int *)p);
+    }
+}
+
+// The dequantised values of N words of codes, as pairs: decoded exactly to binary32, then
+// one RNE multiply by the block scale each (packed).
+template <int FMT, int N>
+__device__ __forceinline__ void qdecode(const uint32_t (&v)[N], float s, uint64_t *d) {
     const uint64_t ss = f2(s, s);
     if (FMT == SHMEMG_FMT_E4M3) {
         // hardware conversion of code pairs to f16 (exact: every E4M3 value is an f16
         // value), then to binary32
 #pragma unroll
-        for (int j = 0; j < 16; j += 2) {
+        for (int j = 0; j < 4 * N; j += 2) {
             const uint16_t pair = (uint16_t)((v[j >> 2] >> (8 * (j & 3))) & 0xFFFFu);
             uint32_t h2;
             asm("cvt.rn.f16x2.e4m3x2 %0, %1;" : "=r"(h2) : "h"(pair));
@@ -113,36 +128,17 @@ __device__ __forceinline__ void qdecode16(uint4 w, float s, uint64_t *d) {
         }
     } else {
 #pragma unroll
-        for (int j = 0; j < 4; j++) d[j] = f2_mul(f2(bf16_decode(v[j] & 0xFFFFu), __uint_as_float(v[j] & 0xFFFF0000u)), ss);
+        for (int j = 0; j < N; j++) d[j] = f2_mul(f2(bf16_decode(v[j] & 0xFFFFu), __uint_as_float(v[j] & 0xFFFF0000u)), ss);
     }
 }
 
-// Wide form of qsum4: elements [e0, e0+E) with E = QWide<FMT>::E, e0 a multiple of E,
-// q_off and d_off 16-byte aligned, e0 + E <= n.  M members' codes and scales are
-// loaded ahead of their accumulation, which stays in team-rank order.
-template <int FMT, int M = 8>
-__device__ __forceinline__ void qsum_wide_acc(const uint8_t *heap, uint64_t H, int pe0, int pstride, int P,
-                                              uint64_t q_off, uint64_t s_off, uint64_t e0, float4 *o);
-
-template <int FMT, int M = 8>
-__device__ __forceinline__ void qsum_wide(uint8_t *heap, uint64_t H, int pe0, int pstride, int P, uint64_t d_off,
-                                          uint64_t q_off, uint64_t s_off, uint64_t e0) {
-    constexpr int E = QWide<FMT>::E;
-    float4 o[E / 4];
-    qsum_wide_acc<FMT, M>(heap, H, pe0, pstride, P, q_off, s_off, e0, o);
-    for (int m = 0; m < P; m++) {
-        float4 *dst = (float4 *)(heap + (uint64_t)(pe0 + m * pstride) * H + d_off + 4 * e0);
-#pragma unroll
-        for (int k = 0; k < E / 4; k++) dst[k] = o[k];
-    }
-}
-
-// The accumulation of qsum_wide: the E compensated sums of elements [e0, e0+E) into o;
-// M members' codes and scales are loaded ahead.
-template <int FMT, int M>
+// The compensated sums of elements [e0, e0+E) over the members into o: e0 a multiple of E,
+// codes aligned to E of them, e0 + E <= n.  M members' codes and scales are loaded ahead
+// of their accumulation, which stays in team-rank order.
+template <int FMT, int M = 8, int E = QWide<FMT>::E>
 __device__ __forceinline__ void qsum_wide_acc(const uint8_t *heap, uint64_t H, int pe0, int pstride, int P,
                                               uint64_t q_off, uint64_t s_off, uint64_t e0, float4 *o) {
-    constexpr int E = QWide<FMT>::E;
+    constexpr int N = QWords<FMT, E>::N;
     constexpr uint64_t QS = FMT == SHMEMG_FMT_E4M3 ? 1 : 2;
     Neu2 acc[E / 2];
 #pragma unroll
@@ -150,24 +146,26 @@ __device__ __forceinline__ void qsum_wide_acc(const uint8_t *heap, uint64_t H, i
     uint64_t d[E / 2];
     int r = 0;
     for (; r + M <= P; r += M) {
-        uint4 w[M];
+        uint32_t w[M][N];
         float sc[M];
 #pragma unroll
         for (int u = 0; u < M; u++) {
             const uint8_t *b = heap + (uint64_t)(pe0 + (r + u) * pstride) * H;
-            w[u] = __ldcg((const uint4 *)(b + q_off + e0 * QS));
+            qload<N>(b + q_off + e0 * QS, w[u]);
             sc[u] = __ldcg((const float *)(b + s_off) + e0 / 128);
         }
 #pragma unroll
         for (int u = 0; u < M; u++) {
-            qdecode16<FMT>(w[u], sc[u], d);
+            qdecode<FMT, N>(w[u], sc[u], d);
 #pragma unroll
             for (int j = 0; j < E / 2; j++) acc[j].add(d[j]);
         }
     }
     for (; r < P; r++) {
         const uint8_t *b0 = heap + (uint64_t)(pe0 + r * pstride) * H;
-        qdecode16<FMT>(__ldcg((const uint4 *)(b0 + q_off + e0 * QS)), __ldcg((const float *)(b0 + s_off) + e0 / 128), d);
+        uint32_t w[N];
+        qload<N>(b0 + q_off + e0 * QS, w);
+        qdecode<FMT, N>(w, __ldcg((const float *)(b0 + s_off) + e0 / 128), d);
 #pragma unroll
         for (int j = 0; j < E / 2; j++) acc[j].add(d[j]);
     }
@@ -186,12 +184,11 @@ __device__ __forceinline__ void qsum_wide_acc(const uint8_t *heap, uint64_t H, i
 // accumulated; before `out` is overwritten thread 0 waits only until every bulk group but
 // the most recent one (the previous chunk's, from the other buffer) has read its source
 // (bulk wait_group.read 1).  Returns with the stores issued as one bulk group.
-template <int FMT, int M = 8>
+template <int FMT, int M = 8, int E = QWide<FMT>::E>
 __device__ __forceinline__ void qsum_chunk_tma(uint8_t *heap, uint64_t H, int pe0, int pstride, int P, uint64_t d_off,
                                                uint64_t q_off, uint64_t s_off, uint64_t c0, float *out) {
-    constexpr int E = QWide<FMT>::E;
     float4 o[E / 4];
-    qsum_wide_acc<FMT, M>(heap, H, pe0, pstride, P, q_off, s_off, c0 + (uint64_t)threadIdx.x * E, o);
+    qsum_wide_acc<FMT, M, E>(heap, H, pe0, pstride, P, q_off, s_off, c0 + (uint64_t)threadIdx.x * E, o);
     if (threadIdx.x == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");  // `out` free again
     __syncthreads();
 #pragma unroll
@@ -209,54 +206,56 @@ __device__ __forceinline__ void qsum_chunk_tma(uint8_t *heap, uint64_t H, int pe
     }
 }
 
-// Dequantised sum of elements [e0, e0+4) over the team members, written to every
-// member's dst.  Vector path: 4 codes and 4 floats per access (aligned offsets).
-template <int FMT>
+// Dequantised sum of elements [e0, e0+4) over the team members, written to every member's
+// dst; of a last group only the elements below n.  vec: the codes are aligned to four of them
+// and d_off to 16 bytes (four codes are then loaded together, past n too: they lie in the
+// same aligned word, inside the partition).  Members are loaded M, or two, ahead either
+// way: one at a time a 128-member team took 115 us for its last few elements (30 teams of up
+// to 4096 elements in one batch 114 -> 18 us).
+template <int FMT, int M = 8>
 __device__ __forceinline__ void qsum4(uint8_t *heap, uint64_t H, int pe0, int pstride, int P, uint64_t d_off,
                                       uint64_t q_off, uint64_t s_off, uint64_t e0, uint64_t n, bool vec) {
-    Neu acc[4];
-#pragma unroll
-    for (int j = 0; j < 4; j++) acc[j] = {0.0f, 0.0f};
-    for (int r = 0; r < P; r++) {
-        const uint8_t *base = heap + (uint64_t)(pe0 + r * pstride) * H;
-        float d[4];
-        if (vec) {
-            const float s = __ldcg((const float *)(base + s_off) + e0 / 128);
-            if (FMT == SHMEMG_FMT_E4M3) {
-                const uint32_t w = __ldcg((const unsigned int *)(base + q_off + e0));
-#pragma unroll
-                for (int j = 0; j < 4; j++) d[j] = __fmul_rn(e4m3_decode((w >> (8 * j)) & 0xFFu), s);
-            } else {
-                const uint2 w = __ldcg((const uint2 *)(base + q_off + 2 * e0));
-                d[0] = __fmul_rn(bf16_decode(w.x & 0xFFFFu), s);
-                d[1] = __fmul_rn(bf16_decode(w.x >> 16), s);
-                d[2] = __fmul_rn(bf16_decode(w.y & 0xFFFFu), s);
-                d[3] = __fmul_rn(bf16_decode(w.y >> 16), s);
-            }
-        } else {
-#pragma unroll
-            for (int j = 0; j < 4; j++) {
-                const uint64_t e = e0 + j;
-                if (e >= n) { d[j] = 0.0f; continue; }
-                const float s = ((const float *)(base + s_off))[e / 128];
-                const float v = FMT == SHMEMG_FMT_E4M3 ? e4m3_decode(base[q_off + e])
-                                                       : bf16_decode(((const uint16_t *)(base + q_off))[e]);
-                d[j] = __fmul_rn(v, s);
-            }
-        }
-#pragma unroll
-        for (int j = 0; j < 4; j++) acc[j].add(d[j]);
-    }
+    float4 o;
     if (vec) {
-        const float4 o = make_float4(acc[0].result(), acc[1].result(), acc[2].result(), acc[3].result());
-        for (int r = 0; r < P; r++) *(float4 *)(heap + (uint64_t)(pe0 + r * pstride) * H + d_off + 4 * e0) = o;
-    } else {
-        for (int r = 0; r < P; r++) {
-            float *dst = (float *)(heap + (uint64_t)(pe0 + r * pstride) * H + d_off);
-#pragma unroll
-            for (int j = 0; j < 4; j++)
-                if (e0 + j < n) dst[e0 + j] = acc[j].result();
+        qsum_wide_acc<FMT, M, 4>(heap, H, pe0, pstride, P, q_off, s_off, e0, &o);
+        if (e0 + 4 <= n) {
+            for (int r = 0; r < P; r++) *(float4 *)(heap + (uint64_t)(pe0 + r * pstride) * H + d_off + 4 * e0) = o;
+            return;
         }
+    } else {
+        constexpr int U = 2;  // members ahead
+        Neu acc[4];
+#pragma unroll
+        for (int j = 0; j < 4; j++) acc[j] = {0.0f, 0.0f};
+        for (int r = 0; r < P; r += U) {
+            float s[U];
+            uint32_t q[U][4];
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                const uint8_t *base = heap + (uint64_t)(pe0 + (r + u < P ? r + u : r) * pstride) * H;
+                s[u] = __ldcg((const float *)(base + s_off) + e0 / 128);
+#pragma unroll
+                for (int j = 0; j < 4; j++) {
+                    const uint64_t e = e0 + j < n ? e0 + j : e0;
+                    q[u][j] = FMT == SHMEMG_FMT_E4M3 ? base[q_off + e] : ((const uint16_t *)(base + q_off))[e];
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < U; u++)
+                if (r + u < P) {
+#pragma unroll
+                    for (int j = 0; j < 4; j++)
+                        acc[j].add(__fmul_rn(FMT == SHMEMG_FMT_E4M3 ? e4m3_decode(q[u][j]) : bf16_decode(q[u][j]), s[u]));
+                }
+        }
+        o = make_float4(acc[0].result(), acc[1].result(), acc[2].result(), acc[3].result());
+    }
+    const float v[4] = {o.x, o.y, o.z, o.w};
+    for (int r = 0; r < P; r++) {
+        float *dst = (float *)(heap + (uint64_t)(pe0 + r * pstride) * H + d_off);
+#pragma unroll
+        for (int j = 0; j < 4; j++)
+            if (e0 + j < n) dst[e0 + j] = v[j];
     }
 }
 

@@ -466,7 +466,7 @@ __device__ uint64_t run_tile(const SvArgs &a, const shmemg_req_t &r0, uint64_t d
                 acc += ck4(w0, 8 * v) + ck4(w1, 8 * v + 4);
             }
             for (uint64_t q = 2 * v1 + threadIdx.x; q < e1 / 4; q += blockDim.x) {
-                qsum4<SHMEMG_FMT_BF16>(heap, H, pe0, 1, P, dst_off, r.src, (uint64_t)r.cond, 4 * q, r.n, true);
+                qsum4<SHMEMG_FMT_BF16, 1>(heap, H, pe0, 1, P, dst_off, r.src, (uint64_t)r.cond, 4 * q, r.n, true);
                 uint4 w = __ldcg((const uint4 *)(heap + (uint64_t)pe0 * H + dst_off + 16 * q));
                 acc += ck4(w, 4 * q);
             }

@@ -111,3 +111,52 @@ def test_collectives_of_ragged_blocks(sg, heapf, P, start, stride, ds, ss):
                     m[q, dst + i * n:dst + (i + 1) * n] = old[p, s:s + n]
             assert first_diff(download(h), want) is None, (op, n)
     sg.team_destroy(team)
+
+
+@pytest.mark.parametrize("tile", [0, 1024, 2048])
+def test_batch_plans_over_ragged_teams(sg, heapf, orc, tile):
+    """The per-team plan (0) and uniform tiles: lengths at the ends of vectors, chunks and
+    tiles, codes on and off their alignments, teams of 1 to 33 members."""
+    world, H = 33, 2 << 20
+    h = heapf(world, H)
+    sizes = [1, 3, 4, 5, 127, 513, 1023, 1024, 1027, 4095, 4096, 5125]
+    kinds = ["i64", "f32", "bf16", "e4m3"]
+    descs, teams = [], []
+    tmp = h.malloc(4 * 6000)
+    x = W.normals_np(8, world * 6000).astype(np.float32).reshape(world, 6000)
+    for p in range(world):
+        h.view(tmp, p, torch.float32, 6000).copy_(torch.from_numpy(x[p]))
+    for k, n in enumerate(sizes):
+        for j, kind in enumerate(kinds):
+            P = (1, 2, 7, 16, 33)[(k + j) % 5]
+            start = (k * 5 + j) % (world - P + 1)
+            shift = (0, 0, 1, 4)[(k + j) % 4]      # elements the source starts off its object
+            qs = {"i64": 8, "f32": 4, "bf16": 2, "e4m3": 1}[kind]
+            src, dst = h.malloc(qs * (n + 8)), h.malloc(8 * (n + 8))
+            so, do = src.offset + shift * qs, dst.offset + (8 if kind == "i64" else 4) * (shift & 1)
+            sc = h.malloc(4 * ((n + 127) // 128))
+            for p in range(world):
+                if kind == "i64":
+                    v = W.uniform_ints_np(k, np.arange(n, dtype=np.uint64) + np.uint64(p * n), -(1 << 40), 1 << 40)
+                    h.view(h.sym(so), p, torch.int64, n).copy_(torch.from_numpy(v))
+                elif kind == "f32":
+                    h.view(h.sym(so), p, torch.float32, n).copy_(torch.from_numpy(x[p, :n]))
+            if qs < 4:
+                sg.quantize(sg.TEAM_WORLD, h.base + so, sc, tmp, 0 if kind == "bf16" else 1, n)
+            fmt = {"bf16": 0, "e4m3": 1}.get(kind, -1)
+            descs.append(sg.CollDesc(start, P, sg.INT64 if kind == "i64" else sg.FLOAT, fmt, n, h.base + do, h.base + so,
+                                     sc.ptr if fmt >= 0 else None))
+            teams.append((kind, (start, 1, P), do, so, sc.offset, fmt, n))
+    torch.cuda.synchronize()
+    init = download(h)
+    b = sg.Batch(descs, sg.Tune(tile, 0, 0, 0) if tile else None)
+    b.launch()
+    got = download(h)
+    b.destroy()
+    ref = orc.Heap(world, H, init)
+    for kind, team, do, so, sco, fmt, n in teams:
+        if fmt >= 0:
+            ref.qsum_reduce(team, do, so, sco, fmt, n)
+        else:
+            ref.reduce(team, do, so, n, W.DT_INT64 if kind == "i64" else W.DT_FLOAT, W.RED_SUM)
+    assert first_diff(got, ref.mem) is None
