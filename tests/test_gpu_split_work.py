@@ -160,3 +160,63 @@ def test_batch_plans_over_ragged_teams(sg, heapf, orc, tile):
         else:
             ref.reduce(team, do, so, n, W.DT_INT64 if kind == "i64" else W.DT_FLOAT, W.RED_SUM)
     assert first_diff(got, ref.mem) is None
+
+
+@pytest.mark.parametrize("fmt", [0, 1])
+@pytest.mark.parametrize("n,qshift", [(128 * 96, 0), (128 * 95 + 77, 1)])
+def test_quantize_near_the_midpoints(sg, heapf, orc, fmt, n, qshift):
+    """Quotients within a few units of the last place of the formats' midpoints, where the
+    codes turn; scales over binary32's whole range, zeros, the smallest numbers."""
+    rng = np.random.RandomState(3 + fmt)
+    if fmt == 1:
+        codes = np.array([orc.e4m3_decode(q) for q in range(127)])
+    else:
+        codes = np.array([orc.bf16_decode(q) for q in range(0x3C00, 0x3F81)])
+    mids = (codes[1:] + codes[:-1]) / 2
+    x = np.zeros((2, 96 * 128), np.float32)
+    for p in range(2):
+        for b in range(96):
+            amax = np.float32(np.ldexp(1 + rng.rand(), rng.randint(-149, 127) if b % 3 == 0 else rng.randint(-20, 20)))
+            s = np.float32(amax / np.float32(448.0)) if fmt == 1 else amax
+            m = mids[rng.randint(0, len(mids), 128)] * rng.choice([-1.0, 1.0], 128)
+            v = (m * np.float64(s) * (1 + rng.randint(-6, 7, 128) * 2.0 ** -25)).astype(np.float32)
+            v[np.abs(v) > amax] = amax
+            v[rng.randint(1, 128, 6)] = [0.0, -0.0, 1e-45, -1e-45, 1.1754944e-38, -amax]
+            v[0] = amax
+            x[p, 128 * b:128 * b + 128] = v
+        x[p, 128 * 7:128 * 8] = 0.0
+    qs = 1 if fmt == 1 else 2
+    h = heapf(2, 1 << 18)
+    src, sc = h.malloc(4 * n), h.malloc(4 * 96)
+    q = h.malloc(qs * (n + 8))
+    for p in range(2):
+        h.view(src, p, torch.float32, n).copy_(torch.from_numpy(x[p, :n]))
+    sg.quantize(sg.TEAM_WORLD, q.ptr + qs * qshift, sc, src, fmt, n)
+    torch.cuda.synchronize()
+    for p in range(2):
+        wq, ws = orc.quantize(x[p, :n], fmt)
+        gs = h.view(sc, p, torch.float32, len(ws)).cpu().numpy()
+        gq = h.view(h.sym(q.offset + qs * qshift), p, torch.uint8, qs * n).cpu().numpy()
+        assert np.array_equal(gs.view(np.uint32), np.asarray(ws, np.float32).view(np.uint32))
+        assert np.array_equal(gq, np.asarray(wq).view(np.uint8).reshape(-1))
+
+
+@pytest.mark.parametrize("fmt", [0, 1])
+@pytest.mark.parametrize("P,n,shift", [(1, 1, 0), (3, 1023, 0), (8, 1024, 0), (17, 5121, 0), (5, 2000, 1), (2, 2 * 608 * 2048 + 1029, 0)])
+def test_qsum_chunk_forms(sg, heapf, orc, fmt, P, n, shift):
+    """Chunks of 4 and 8 elements per thread, their tails, codes off their alignment."""
+    qs = 1 if fmt == 1 else 2
+    nb = (n + 127) // 128
+    H = ((qs + 4) * (n + 512) + 4 * nb + 65536 + 4 * (n + 512)) // 4096 * 4096 + 4096
+    h = heapf(P, H)
+    src, q, sc, dst = h.malloc(4 * n), h.malloc(qs * (n + 8)), h.malloc(4 * nb), h.malloc(4 * n)
+    x = W.normals_np(6, P * n).astype(np.float32).reshape(P, n)
+    for p in range(P):
+        h.view(src, p, torch.float32, n).copy_(torch.from_numpy(x[p]))
+    sg.quantize(sg.TEAM_WORLD, q.ptr + qs * shift, sc, src, fmt, n)
+    torch.cuda.synchronize()
+    init = download(h)
+    sg.qsum_reduce(sg.TEAM_WORLD, dst, q.ptr + qs * shift, sc, fmt, n)
+    ref = orc.Heap(P, H, init)
+    ref.qsum_reduce((0, 1, P), dst.offset, q.offset + qs * shift, sc.offset, fmt, n)
+    assert first_diff(download(h), ref.mem) is None
