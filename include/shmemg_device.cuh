@@ -818,58 +818,65 @@ template <> __device__ __forceinline__ float shmemg_comb<float>(float a, float b
     return op == SHMEMG_MAX ? (b > a ? b : a) : (b < a ? b : a);  /* sums use the tree */
 }
 
-/* Slice-owner reduce of vectors [v0, v1) (V = T or a 16-byte vector of T): each thread
- * of g owns vectors, reads them from the P members pe0 + r*pstride, combines (integer
- * sums wrap; float sums by the rank-pairwise tree; max/min exact) and writes the result
- * to every member's dst. */
+/* The combined value of one vector (V = T or a 16-byte vector of T) at byte offset `off` of the
+ * P members pe0 + r*pstride: integer sums wrap; float sums by the rank-pairwise tree; max/min
+ * exact. */
+template <typename T, typename V, int OP, int TREE_MAXB = 5>
+static __device__ __forceinline__ V shmemg_d_reduce_vec(const uint8_t *heap, uint64_t H, int pe0, int pstride, int P,
+                                                        uint64_t off) {
+    constexpr int NL = sizeof(V) / sizeof(T);
+    V acc;
+    if constexpr (OP == SHMEMG_SUM && std::is_floating_point<T>::value) {
+        acc = shmemg_tree_sum<V, TREE_MAXB>(heap, H, pe0, pstride, P, off);
+    } else {
+        acc = shmemg_ld_cg((const V *)(heap + (uint64_t)pe0 * H + off));
+        int r = 1;
+        for (; r + 7 < P; r += 8) {  /* eight members' loads in flight */
+            V x[8];
+#pragma unroll
+            for (int u = 0; u < 8; u++) x[u] = shmemg_ld_cg((const V *)(heap + (uint64_t)(pe0 + (r + u) * pstride) * H + off));
+#pragma unroll
+            for (int u = 0; u < 8; u++)
+#pragma unroll
+                for (int l = 0; l < NL; l++) {
+                    T &s = reinterpret_cast<T *>(&acc)[l];
+                    s = shmemg_comb<T>(s, reinterpret_cast<T *>(&x[u])[l], OP);
+                }
+        }
+        for (; r + 3 < P; r += 4) {
+            V a = shmemg_ld_cg((const V *)(heap + (uint64_t)(pe0 + r * pstride) * H + off));
+            V b = shmemg_ld_cg((const V *)(heap + (uint64_t)(pe0 + (r + 1) * pstride) * H + off));
+            V d = shmemg_ld_cg((const V *)(heap + (uint64_t)(pe0 + (r + 2) * pstride) * H + off));
+            V e = shmemg_ld_cg((const V *)(heap + (uint64_t)(pe0 + (r + 3) * pstride) * H + off));
+#pragma unroll
+            for (int l = 0; l < NL; l++) {
+                T &s = reinterpret_cast<T *>(&acc)[l];
+                s = shmemg_comb<T>(s, reinterpret_cast<T *>(&a)[l], OP);
+                s = shmemg_comb<T>(s, reinterpret_cast<T *>(&b)[l], OP);
+                s = shmemg_comb<T>(s, reinterpret_cast<T *>(&d)[l], OP);
+                s = shmemg_comb<T>(s, reinterpret_cast<T *>(&e)[l], OP);
+            }
+        }
+        for (; r < P; r++) {
+            V a = shmemg_ld_cg((const V *)(heap + (uint64_t)(pe0 + r * pstride) * H + off));
+#pragma unroll
+            for (int l = 0; l < NL; l++) {
+                T &s = reinterpret_cast<T *>(&acc)[l];
+                s = shmemg_comb<T>(s, reinterpret_cast<T *>(&a)[l], OP);
+            }
+        }
+    }
+    return acc;
+}
+
+/* Slice-owner reduce of vectors [v0, v1): each thread of g owns vectors, combines them over
+ * the members and writes the result to every member's dst. */
 template <typename T, typename V, int OP, int TREE_MAXB = 5>
 static __device__ __forceinline__ void shmemg_d_reduce_vecs(shmemg_group g, uint8_t *heap, uint64_t H, int pe0,
                                                            int pstride, int P, uint64_t dst_off, uint64_t src_off,
                                                            uint64_t v0, uint64_t v1) {
-    constexpr int NL = sizeof(V) / sizeof(T);
     for (uint64_t vi = v0 + g.rank; vi < v1; vi += g.size) {
-        const uint64_t off = src_off + vi * sizeof(V);
-        V acc;
-        if constexpr (OP == SHMEMG_SUM && std::is_floating_point<T>::value) {
-            acc = shmemg_tree_sum<V, TREE_MAXB>(heap, H, pe0, pstride, P, off);
-        } else {
-            acc = shmemg_ld_cg((const V *)(heap + (uint64_t)pe0 * H + off));
-            int r = 1;
-            for (; r + 7 < P; r += 8) {  /* eight members' loads in flight */
-                V x[8];
-#pragma unroll
-                for (int u = 0; u < 8; u++) x[u] = shmemg_ld_cg((const V *)(heap + (uint64_t)(pe0 + (r + u) * pstride) * H + off));
-#pragma unroll
-                for (int u = 0; u < 8; u++)
-#pragma unroll
-                    for (int l = 0; l < NL; l++) {
-                        T &s = reinterpret_cast<T *>(&acc)[l];
-                        s = shmemg_comb<T>(s, reinterpret_cast<T *>(&x[u])[l], OP);
-                    }
-            }
-            for (; r + 3 < P; r += 4) {
-                V a = shmemg_ld_cg((const V *)(heap + (uint64_t)(pe0 + r * pstride) * H + off));
-                V b = shmemg_ld_cg((const V *)(heap + (uint64_t)(pe0 + (r + 1) * pstride) * H + off));
-                V d = shmemg_ld_cg((const V *)(heap + (uint64_t)(pe0 + (r + 2) * pstride) * H + off));
-                V e = shmemg_ld_cg((const V *)(heap + (uint64_t)(pe0 + (r + 3) * pstride) * H + off));
-#pragma unroll
-                for (int l = 0; l < NL; l++) {
-                    T &s = reinterpret_cast<T *>(&acc)[l];
-                    s = shmemg_comb<T>(s, reinterpret_cast<T *>(&a)[l], OP);
-                    s = shmemg_comb<T>(s, reinterpret_cast<T *>(&b)[l], OP);
-                    s = shmemg_comb<T>(s, reinterpret_cast<T *>(&d)[l], OP);
-                    s = shmemg_comb<T>(s, reinterpret_cast<T *>(&e)[l], OP);
-                }
-            }
-            for (; r < P; r++) {
-                V a = shmemg_ld_cg((const V *)(heap + (uint64_t)(pe0 + r * pstride) * H + off));
-#pragma unroll
-                for (int l = 0; l < NL; l++) {
-                    T &s = reinterpret_cast<T *>(&acc)[l];
-                    s = shmemg_comb<T>(s, reinterpret_cast<T *>(&a)[l], OP);
-                }
-            }
-        }
+        const V acc = shmemg_d_reduce_vec<T, V, OP, TREE_MAXB>(heap, H, pe0, pstride, P, src_off + vi * sizeof(V));
         const uint64_t doff = dst_off + vi * sizeof(V);
         for (int r = 0; r < P; r++) *(V *)(heap + (uint64_t)(pe0 + r * pstride) * H + doff) = acc;
     }

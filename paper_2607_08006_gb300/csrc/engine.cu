@@ -365,41 +365,76 @@ struct Red {
     uint64_t H;
     int start, stride, size, gstride;
     uint64_t dst_off, src_off;
-    uint64_t nvec;        // vectors (V) per member
+    uint64_t nvec;        // vectors (V) per member, a partial last one included
+    uint32_t tail;        // elements of a partial last vector (0: it is whole)
     uint64_t chunk_vec;
     uint64_t nitems;
     uint32_t rb_chunk, rb_stages;  // k_reduce_bulk: bytes per member per chunk, ring stages
 };
 
-template <typename T, typename V, int OP>
-__global__ void __launch_bounds__(RED_THREADS) k_reduce(Red x) {
-    const int pe0 = x.start + blockIdx.y * x.gstride;
-    const shmemg_group g = {threadIdx.x, blockDim.x};
-    for (uint64_t item = blockIdx.x; item < x.nitems; item += gridDim.x) {
-        const uint64_t v0 = item * x.chunk_vec;
-        const uint64_t v1 = v0 + x.chunk_vec < x.nvec ? v0 + x.chunk_vec : x.nvec;
-        shmemg_d_reduce_vecs<T, V, OP>(g, x.heap, x.H, pe0, x.stride, x.size, x.dst_off, x.src_off, v0, v1);
+// The result of vector vi into the dst of members r0, r0 + step, ...  A length that is no
+// multiple of a vector ends in a partial one: its loads read it whole (the bytes past the
+// object lie in the same 16-byte granule, inside the partition), its stores write the
+// elements of the object only.
+template <typename T, typename V>
+__device__ __forceinline__ void red_store(const Red &x, int pe0, int r0, int step, uint64_t vi, const V &v) {
+    uint8_t *d = x.heap + (uint64_t)(pe0 + r0 * x.stride) * x.H + x.dst_off + vi * sizeof(V);
+    const uint64_t next = (uint64_t)(step * x.stride) * x.H;
+    if (sizeof(V) == sizeof(T) || x.tail == 0 || vi != x.nvec - 1) {
+        for (int r = r0; r < x.size; r += step, d += next) *(V *)d = v;
+    } else {
+        for (int r = r0; r < x.size; r += step, d += next)
+#pragma unroll
+            for (int l = 0; l < (int)(sizeof(V) / sizeof(T)); l++)
+                if (l < (int)x.tail) ((T *)d)[l] = reinterpret_cast<const T *>(&v)[l];
     }
 }
 
-// Integer sum / max / min of few vectors per member: G threads share a 16-byte vector,
-// each combining the members sub, sub + G, ... (integer combining is exact in any order),
-// the G partial results meet by warp shuffles, and the G threads store the result to every
-// G-th member.  A launch of few vectors keeps G times as many loads in flight and needs
-// P / (8G) dependent rounds instead of P / 8.  Requires P >= G.
+template <typename T, typename V, int OP>
+__global__ void __launch_bounds__(RED_THREADS) k_reduce(Red x) {
+    const int pe0 = x.start + blockIdx.y * x.gstride;
+    for (uint64_t item = blockIdx.x; item < x.nitems; item += gridDim.x) {
+        const uint64_t v0 = item * x.chunk_vec;
+        const uint64_t v1 = v0 + x.chunk_vec < x.nvec ? v0 + x.chunk_vec : x.nvec;
+        for (uint64_t vi = v0 + threadIdx.x; vi < v1; vi += RED_THREADS) {
+            const V acc = shmemg_d_reduce_vec<T, V, OP>(x.heap, x.H, pe0, x.stride, x.size, x.src_off + vi * sizeof(V));
+            red_store<T, V>(x, pe0, 0, 1, vi, acc);
+        }
+    }
+}
+
+// Reductions of few vectors per member: G threads share a 16-byte vector, the G partial
+// results meet by warp shuffles, and the G threads store the result to every G-th member.
+// A launch of few vectors keeps G times as many loads in flight and needs P / (8G)
+// dependent rounds instead of P / 8.  Requires P >= G.
+//   Integers: thread g combines members g, g + G, ... (exact in any order).
+//   Floats: thread g combines the aligned rank block [g*B, (g+1)*B), B the power of two with
+// ceil(P/B) <= G blocks.  The rank-pairwise tree pairs within such blocks first (a value
+// carried up stays last in its block), so its upper levels are the same tree over the blocks'
+// values.  max / min: comparisons in rank order, first of equals; a NaN of rank 0 stays and
+// any other is passed over, so a block other than the first starts at its first number.
 template <typename T, typename V, int OP, int G>
 __global__ void __launch_bounds__(RED_THREADS) k_reduce_split(Red x) {
     constexpr int NL = sizeof(V) / sizeof(T);
+    constexpr bool FLT = std::is_floating_point<T>::value;
     const int pe0 = x.start + blockIdx.y * x.gstride;
     const int sub = (int)(threadIdx.x % G);
     const uint64_t per_cta = blockDim.x / G;
+    int B = 1;  // floats: ranks per block, blocks
+    while (B * G < x.size) B *= 2;
+    const int nblk = (x.size + B - 1) / B;
     auto member = [&](int r, uint64_t off) {
         return shmemg_ld_cg((const V *)(x.heap + (uint64_t)(pe0 + r * x.stride) * x.H + off));
     };
     auto comb = [&](V &a, const V &b) {
 #pragma unroll
-        for (int l = 0; l < NL; l++)
-            reinterpret_cast<T *>(&a)[l] = shmemg_comb<T>(reinterpret_cast<T *>(&a)[l], reinterpret_cast<const T *>(&b)[l], OP);
+        for (int l = 0; l < NL; l++) {
+            T &s = reinterpret_cast<T *>(&a)[l];
+            const T v = reinterpret_cast<const T *>(&b)[l];
+            if constexpr (!FLT) s = shmemg_comb<T>(s, v, OP);
+            else if constexpr (OP == SHMEMG_SUM) s = __fadd_rn(s, v);
+            else s = sub > 0 && s != s ? v : shmemg_comb<T>(s, v, OP);
+        }
     };
     // warp-uniform loop: every lane runs every round (lanes past the end load vector 0 and
     // store nothing), so the shuffles always see full warps
@@ -407,33 +442,46 @@ __global__ void __launch_bounds__(RED_THREADS) k_reduce_split(Red x) {
         const uint64_t vi = vb + threadIdx.x / G;
         const bool act = vi < x.nvec;
         const uint64_t off = x.src_off + (act ? vi : 0) * sizeof(V);
-        V acc = member(sub, off);
-        int r = sub + G;
-        for (; r + 7 * G < x.size; r += 8 * G) {  // eight members' loads in flight
-            V v[8];
+        const int r0 = FLT ? sub * B : sub, step = FLT ? 1 : G, r1 = FLT && r0 + B < x.size ? r0 + B : x.size;
+        V acc{};
+        if (FLT && OP == SHMEMG_SUM) {
+            if constexpr (FLT)
+                if (r0 < r1) acc = shmemg_tree_sum<V>(x.heap, x.H, pe0 + r0 * x.stride, x.stride, r1 - r0, off);
+        } else if (r0 < r1) {
+            acc = member(r0, off);
+            int r = r0 + step;
+            for (; r + 7 * step < r1; r += 8 * step) {  // eight members' loads in flight
+                V v[8];
 #pragma unroll
-            for (int u = 0; u < 8; u++) v[u] = member(r + u * G, off);
+                for (int u = 0; u < 8; u++) v[u] = member(r + u * step, off);
 #pragma unroll
-            for (int u = 0; u < 8; u++) comb(acc, v[u]);
+                for (int u = 0; u < 8; u++) comb(acc, v[u]);
+            }
+            for (; r < r1; r += step) comb(acc, member(r, off));
         }
-        for (; r < x.size; r += G) comb(acc, member(r, off));
-#pragma unroll
-        for (int m = G / 2; m > 0; m >>= 1) {
+        auto shuffle = [&](auto get) {
             V o;
             if constexpr (sizeof(T) == 8) {
 #pragma unroll
-                for (int l = 0; l < NL; l++)
-                    reinterpret_cast<long long *>(&o)[l] = __shfl_xor_sync(0xffffffffu, reinterpret_cast<long long *>(&acc)[l], m);
+                for (int l = 0; l < NL; l++) reinterpret_cast<long long *>(&o)[l] = get(reinterpret_cast<long long *>(&acc)[l]);
             } else {
 #pragma unroll
-                for (int l = 0; l < NL; l++)
-                    reinterpret_cast<int *>(&o)[l] = __shfl_xor_sync(0xffffffffu, reinterpret_cast<int *>(&acc)[l], m);
+                for (int l = 0; l < NL; l++) reinterpret_cast<int *>(&o)[l] = get(reinterpret_cast<int *>(&acc)[l]);
             }
-            comb(acc, o);
+            return o;
+        };
+        if constexpr (FLT) {  // the blocks' values level by level, the last of an odd number carried up
+#pragma unroll
+            for (int m = 1; m < G; m <<= 1) {
+                const V o = shuffle([&](auto v) { return __shfl_down_sync(0xffffffffu, v, m, G); });
+                if (sub % (2 * m) == 0 && sub + m < nblk) comb(acc, o);
+            }
+            acc = shuffle([&](auto v) { return __shfl_sync(0xffffffffu, v, 0, G); });
+        } else {
+#pragma unroll
+            for (int m = G / 2; m > 0; m >>= 1) comb(acc, shuffle([&](auto v) { return __shfl_xor_sync(0xffffffffu, v, m); }));
         }
-        if (act)
-            for (int q = sub; q < x.size; q += G)
-                *(V *)(x.heap + (uint64_t)(pe0 + q * x.stride) * x.H + x.dst_off + vi * sizeof(V)) = acc;
+        if (act) red_store<T, V>(x, pe0, sub, G, vi, acc);
     }
 }
 
@@ -547,9 +595,7 @@ __global__ void __launch_bounds__(RB_THREADS, 1) k_reduce_bulk(Red x, uint8_t *s
         if (col < nc) {
             V acc = pb[col];
             for (uint32_t q = 1; q < nparts; q++) comb(acc, pb[q * ncol + col]);
-            const uint64_t doff = x.dst_off + c * C + (uint64_t)col * 16;
-            for (int r = (int)part; r < P; r += (int)nparts)
-                *(V *)(x.heap + (uint64_t)(pe0 + r * x.stride) * x.H + doff) = acc;
+            red_store<T, V>(x, pe0, (int)part, (int)nparts, c * (C / 16) + col, acc);
         }
     }
 }
@@ -746,7 +792,9 @@ static bool rb_shape(int P, uint32_t *chunk, uint32_t *stages) {
 
 template <typename V, typename T, int OP>
 static int launch_red_v(Red r, int ngroups, cudaStream_t s) {
-    r.nvec /= (sizeof(V) / sizeof(T));
+    constexpr uint64_t NL = sizeof(V) / sizeof(T);
+    r.tail = (uint32_t)(r.nvec % NL);
+    r.nvec = (r.nvec + NL - 1) / NL;
     r.chunk_vec = (uint64_t)RED_THREADS * RED_U;
     r.nitems = (r.nvec + r.chunk_vec - 1) / r.chunk_vec;
     if (r.nitems == 0) return SHMEMG_SUCCESS;
@@ -761,8 +809,10 @@ static int launch_red_v(Red r, int ngroups, cudaStream_t s) {
             k_reduce_bulk<T, V, OP><<<grid, RB_THREADS, RB_SMEM, s>>>(r, st().base, st().timeout_ns);
             return cuda_rc(cudaGetLastError());
         }
-        // integer teams with too few vectors to fill the GPU one thread each: several
-        // threads per vector (k_reduce_split)
+    }
+    if constexpr (sizeof(V) == 16) {
+        // teams with too few vectors to fill the GPU one thread each: several threads per
+        // vector (k_reduce_split)
         const int G = r.size >= 32 ? 8 : r.size >= 8 ? 4 : 1;
         const void *kf = G == 8 ? (const void *)k_reduce_split<T, V, OP, 8> : (const void *)k_reduce_split<T, V, OP, 4>;
         if (G > 1) {
@@ -780,11 +830,19 @@ static int launch_red_v(Red r, int ngroups, cudaStream_t s) {
     }
     const void *kfn = (const void *)k_reduce<T, V, OP>;
     const uint64_t cap = (uint64_t)ctas_for(kfn, RED_THREADS, 0);
-    if (r.nitems * (uint64_t)ngroups < cap) {  // too few items for the resident CTAs: one vector per thread
+    // One vector per thread where that gives the resident CTAs less than two, or at least three
+    // rounds: then every CTA takes one item and the queue is left to the hardware (fp32 sum,
+    // 24 PEs x 4 M: 137 us with resident CTAs taking two vectors a thread in turn, 118 so; int32,
+    // 20 PEs x 3 M, 3.2 rounds: 81 and 75; int64, 30 PEs x 1.5 M, 3.2 rounds: 114 and 115).  In
+    // between resident CTAs share the items evenly (int32, 30 PEs x 1 Mi, 1.1 rounds: 43 us
+    // against 49).
+    const uint64_t ones = (r.nvec + RED_THREADS - 1) / RED_THREADS;
+    const bool queue = ones * (uint64_t)ngroups >= 3 * cap && ones < (1u << 30);
+    if (queue || r.nitems * (uint64_t)ngroups < cap) {
         r.chunk_vec = RED_THREADS;
-        r.nitems = (r.nvec + r.chunk_vec - 1) / r.chunk_vec;
+        r.nitems = ones;
     }
-    dim3 grid((unsigned)balanced_grid(r.nitems, cap, ngroups), (unsigned)ngroups);
+    dim3 grid((unsigned)(queue ? r.nitems : balanced_grid(r.nitems, cap, ngroups)), (unsigned)ngroups);
     k_reduce<T, V, OP><<<grid, RED_THREADS, 0, s>>>(r);
     return cuda_rc(cudaGetLastError());
 }
@@ -970,7 +1028,7 @@ int shmemg_reduce(shmemg_team_t team, void *dst, const void *src, uint64_t nelem
     r.dst_off = doff;
     r.src_off = soff;
     r.nvec = nelems;
-    bool v16 = ((doff | soff | (nelems * es)) & 15) == 0;
+    bool v16 = ((doff | soff) & 15) == 0;
     cudaStream_t s = to_stream(stream);
     int g = t.ngroups;
 #define SHMEMG_RED(T, V) \

@@ -220,3 +220,54 @@ def test_qsum_chunk_forms(sg, heapf, orc, fmt, P, n, shift):
     ref = orc.Heap(P, H, init)
     ref.qsum_reduce((0, 1, P), dst.offset, q.offset + qs * shift, sc.offset, fmt, n)
     assert first_diff(download(h), ref.mem) is None
+
+
+@pytest.mark.parametrize("dt,op", [("int32", 0), ("int64", 1), ("int64", 0), ("float", 0), ("float", 1), ("float", 2)])
+@pytest.mark.parametrize("P,start,stride", [(1, 0, 1), (7, 3, 2), (8, 0, 1), (24, 1, 2), (33, 2, 1), (50, 0, 1), (64, 0, 1)])
+def test_reduce_ragged_lengths(sg, heapf, orc, dt, op, P, start, stride):
+    """Partial last vectors in every form -- several threads per vector, one, the bulk ring --
+    in place and not: nothing past the object changes."""
+    es = 8 if dt == "int64" else 4
+    sizes = [1, 3, 5, 1023, 4099] + ([32771] if P in (24, 50) else []) + ([300001] if P == 8 else [])
+    npes, n_max = 64, max(sizes)
+    H = (2 * es * (n_max + 64) + 4095) // 4096 * 4096
+    h = heapf(npes, H)
+    team = sg.team_split_strided(sg.TEAM_WORLD, start, stride, P)
+    code = {"int32": sg.INT32, "int64": sg.INT64, "float": sg.FLOAT}[dt]
+    for k, n in enumerate(sizes):
+        init = random_heap(npes, H, 40 + k)
+        if dt == "float":
+            init = W.normals_np(9 + k, npes * H // 4).astype(np.float32).view(np.uint8).copy()
+        src, dst = 256, (256 if k % 2 else 256 + (es * n + 271) // 16 * 16)
+        upload(h, init)
+        sg.reduce(team, h.base + dst, h.base + src, n, code, op)
+        ref = orc.Heap(npes, H, init)
+        ref.reduce((start, stride, P), dst, src, n, {"int32": W.DT_INT32, "int64": W.DT_INT64, "float": W.DT_FLOAT}[dt],
+                   (W.RED_SUM, W.RED_MAX, W.RED_MIN)[op])
+        assert first_diff(download(h), ref.mem) is None, n
+    sg.team_destroy(team)
+
+
+@pytest.mark.parametrize("op", [1, 2])
+@pytest.mark.parametrize("P", [7, 8, 24, 41, 64])
+def test_reduce_float_extrema_of_special_values(sg, heapf, op, P):
+    """NaN, infinities and signed zeros: a member's value replaces the running one only where
+    it compares greater (less), members in rank order, whatever threads share a vector."""
+    n = 2000
+    h = heapf(64, 1 << 16)
+    rng = np.random.RandomState(P)
+    x = rng.choice(np.array([0.0, -0.0, np.nan, np.inf, -np.inf, 1.5, -2.0], np.float32), (64, n))
+    src, dst = h.malloc(4 * n), h.malloc(4 * n)
+    for p in range(64):
+        h.view(src, p, torch.float32, n).copy_(torch.from_numpy(x[p]))
+    team = sg.team_split_strided(sg.TEAM_WORLD, 0, 1, P)
+    sg.reduce(team, dst, src, n, sg.FLOAT, op)
+    want = x[0].copy()
+    with np.errstate(invalid="ignore"):
+        for p in range(1, P):
+            take = x[p] > want if op == 1 else x[p] < want
+            want[take] = x[p][take]
+    for p in (0, P - 1):
+        got = h.view(dst, p, torch.float32, n).cpu().numpy()
+        assert np.array_equal(got.view(np.uint32), want.view(np.uint32))
+    sg.team_destroy(team)
