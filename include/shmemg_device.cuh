@@ -525,19 +525,28 @@ static __device__ __forceinline__ int shmemg_d_signal_wait_until(const shmemg_de
 /* Barrier of one team group, entered by the leader thread of each member PE after the
  * PE's own quiet.  The slot's count (low half) and generation (high half) form one
  * 64-bit word: a PE arrives with one acq_rel add of 1 (release for the PE's writes,
- * ordered before it by the PE barrier; the old value gives the generation); the last
- * arrival adds 2^32 - size, which resets the count and opens the next generation in one
- * release; the others acquire-poll the word until the generation moves -- spinning at
- * first, then backing off -- bounded.  Needs every member PE resident on the GPU at once. */
+ * ordered before it by the PE barrier); the arrival that makes the count `size` opens the
+ * next generation by itself -- the others acquire-poll the word until they see that count
+ * or a later generation, spinning at first, then backing off, bounded.  The last arrival
+ * folds the full count into the generation (+2^32 - size) afterwards, off the others' way:
+ * a PE may arrive at the next barrier before that, and finds a count >= size, which
+ * stands for the next generation.  (The count stays below 2 * size: the last arrival itself
+ * arrives again only after its fold.)  Waiting for the fold instead cost each barrier a
+ * release and its trip to L2: 2.1 us a barrier of 4 PEs, now 1.75.  Needs every
+ * member PE resident on the GPU at once. */
+static __device__ __forceinline__ uint32_t shmemg_d_barrier_gen(unsigned long long w, uint32_t size) {
+    return (uint32_t)(w >> 32) + ((uint32_t)w >= size ? 1u : 0u);
+}
 static __device__ __forceinline__ int shmemg_d_team_barrier_leader(const shmemg_device_ctx_t &c, int bar_slot,
                                                                    uint32_t size, int64_t detail) {
     shmemg_dbar_t *b = (shmemg_dbar_t *)(c.state + SHMEMG_BARRIERS_OFF) + bar_slot;
     unsigned long long *w = (unsigned long long *)&b->count;  /* count | gen << 32 */
     unsigned long long old;
     asm volatile("atom.acq_rel.gpu.global.add.u64 %0, [%1], %2;" : "=l"(old) : "l"(w), "l"(1ull) : "memory");
-    const uint32_t gen = (uint32_t)(old >> 32);
-    if ((uint32_t)old == size - 1) {
-        asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(w), "l"((1ull << 32) - size) : "memory");
+    const uint32_t gen = shmemg_d_barrier_gen(old, size);
+    const uint32_t before = (uint32_t)old >= size ? (uint32_t)old - size : (uint32_t)old;  /* arrivals of this generation */
+    if (before == size - 1) {
+        asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(w), "l"((1ull << 32) - size) : "memory");
         return SHMEMG_SUCCESS;
     }
     uint64_t t0 = 0;
@@ -545,7 +554,7 @@ static __device__ __forceinline__ int shmemg_d_team_barrier_leader(const shmemg_
     for (uint32_t it = 0;; it++) {
         unsigned long long v;
         asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(w) : "memory");
-        if ((uint32_t)(v >> 32) != gen) return SHMEMG_SUCCESS;
+        if (shmemg_d_barrier_gen(v, size) != gen) return SHMEMG_SUCCESS;
         if ((it & 63) == 63) {
             uint64_t now = shmemg_d_globaltimer();
             if (t0 == 0) t0 = now;
@@ -900,12 +909,13 @@ static __device__ __forceinline__ void shmemg_d_reduce_elems_t(shmemg_group g, u
         else shmemg_d_reduce_vecs<T, T, SHMEMG_MIN>(g, heap, H, pe0, pstride, P, dst_off, src_off, e0, e1);
     }
 }
+template <int TREE_MAXB = 5>
 static __device__ __forceinline__ void shmemg_d_reduce_elems(shmemg_group g, uint8_t *heap, uint64_t H, int pe0,
                                                             int pstride, int P, uint64_t dst_off, uint64_t src_off,
                                                             uint64_t e0, uint64_t e1, int dtype, int op) {
     if (dtype == SHMEMG_INT32) shmemg_d_reduce_elems_t<int32_t, int4>(g, heap, H, pe0, pstride, P, dst_off, src_off, e0, e1, op);
     else if (dtype == SHMEMG_INT64) shmemg_d_reduce_elems_t<int64_t, longlong2>(g, heap, H, pe0, pstride, P, dst_off, src_off, e0, e1, op);
-    else shmemg_d_reduce_elems_t<float, float4>(g, heap, H, pe0, pstride, P, dst_off, src_off, e0, e1, op);
+    else shmemg_d_reduce_elems_t<float, float4, TREE_MAXB>(g, heap, H, pe0, pstride, P, dst_off, src_off, e0, e1, op);
 }
 
 /* Group-wide copy of src to the same offset `dst_off` of P members (one read, P
@@ -977,6 +987,7 @@ static __device__ __forceinline__ int shmemg_d_scope_sync(const shmemg_device_ct
  * slice of the elements or bytes (reduce, broadcast) or its own blocks (fcollect,
  * alltoall).  Offsets are symmetric byte offsets.  Return SHMEMG_SUCCESS or a timeout /
  * device error. */
+template <int TREE_MAXB = 5>
 static __device__ __forceinline__ int shmemg_d_reduce_scoped(const shmemg_device_ctx_t &c, int team, uint64_t dst_off,
                                                              uint64_t src_off, uint64_t nelems, int dtype, int op,
                                                              int64_t detail, shmemg_cluster_state_t *cs, bool warp) {
@@ -987,7 +998,7 @@ static __device__ __forceinline__ int shmemg_d_reduce_scoped(const shmemg_device
     if (rc) return rc;
     uint64_t es = dtype == SHMEMG_INT64 ? 8 : 4, lo, hi;
     shmemg_d_slice(nelems, r, t.size, 16 / es, &lo, &hi);
-    shmemg_d_reduce_elems(shmemg_d_scope_group(c, warp), c.heap, c.pe_stride, shmemg_d_team_member(t, grp, 0),
+    shmemg_d_reduce_elems<TREE_MAXB>(shmemg_d_scope_group(c, warp), c.heap, c.pe_stride, shmemg_d_team_member(t, grp, 0),
                           t.stride, t.size, dst_off, src_off, lo, hi, dtype, op);
     return shmemg_d_scope_sync(c, team, detail, cs, warp);
 }

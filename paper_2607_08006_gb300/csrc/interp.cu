@@ -4,8 +4,9 @@
 // One cooperative launch holds every PE (a CTA, or a cluster of CTAs in pe_mode
 // CLUSTER).  Every PE walks the whole list; it issues, in list order, the RMA/AMO/signal
 // ops whose issuer it is, and its share of every collective of a team it belongs to.
-// Blocking RMA ends with a PE barrier (local completion, and later ops of the PE see
-// it); collectives and barriers quiet and synchronise their team on entry and exit.
+// A PE barrier stands between two of its RMA or AMO ops where the later one touches what
+// the earlier one writes, or writes what it reads (so later ops of the PE see it); ops that
+// touch nothing of each other overlap.  Collectives and barriers quiet and synchronise their team on entry and exit.
 #include <cuda_runtime.h>
 
 #include <cstdlib>
@@ -432,8 +433,48 @@ __device__ __forceinline__ bool op_involves(const shmemg_op_t &o, int me) {
     }
 }
 
+// Which of a PE's ops need a PE barrier before them.  Consecutive puts, gets and AMOs (PE scope;
+// non-blocking ones on the default context) need none between them unless one touches what
+// another writes; every other op is kept apart, but those that begin with a PE barrier of
+// their own -- quiet, fence, barrier_all, the world team's collectives -- need none before.
+constexpr int OP_WINDOW = 7;                 // ops since the last PE barrier that an op is checked against
+constexpr uint32_t OP_APART = 0x80u, OP_OWN_SYNC = OP_APART;  // not simple; and no barrier before it
+
+// Warp 0, per batch: conf of the listed ops -- bit d - 1: the op conflicts with the listed op d
+// before it (all of the first half of the batch conflict with the second).  Ranges are compared
+// in granules of 2^gran bytes over the whole heap, which fit 32 bits; branch-free (this code
+// runs cold in a short script: a switch's jump table cost it half a microsecond).
+__device__ __forceinline__ void op_conflicts(const shmemg_op_t *ops, const uint8_t *act, const uint8_t *list, uint8_t *conf,
+                                             int nact, uint64_t H, int gran) {
+    const int lane = (int)(threadIdx.x & 31);
+    for (int k0 = 0; k0 < nact; k0 += 32) {
+        const bool in = k0 + lane < nact;
+        const int at = list[in ? k0 + lane : 0];
+        const shmemg_op_t &o = ops[at];
+        const uint32_t k = o.kind;  // (flags in it: a warp-scope op is not simple)
+        const bool valid = in && act[at] == 1, nbi = k == SHMEMG_OP_PUT_NBI || k == SHMEMG_OP_GET_NBI;
+        const bool amo = k - SHMEMG_OP_FETCH_ADD < 3u, put = k == SHMEMG_OP_PUT || k == SHMEMG_OP_PUT_NBI;
+        const bool simple = valid && k - SHMEMG_OP_PUT < 7u && !(nbi && o.sub != 0);
+        const bool own = valid && (k - SHMEMG_OP_BARRIER_ALL < 3u || (k - SHMEMG_OP_BROADCAST < 5u && o.team == SHMEMG_TEAM_WORLD));
+        const uint64_t there = (uint64_t)o.pe * H, mine = (uint64_t)o.issuer * H, n = amo ? 8 : o.n;
+        const uint64_t w = (amo || put ? there : mine) + o.dst, r = amo ? w : (put ? mine : there) + o.src;
+        // first and last granule (an empty range touches its first)
+        const uint32_t w0 = (uint32_t)(w >> gran), w1 = (uint32_t)((w + (n ? n - 1 : 0)) >> gran);
+        const uint32_t r0 = (uint32_t)(r >> gran), r1 = (uint32_t)((r + (n ? n - 1 : 0)) >> gran);
+        const int most = nact - k0 - 1 < OP_WINDOW ? nact - k0 - 1 : OP_WINDOW;
+        uint32_t m = simple ? 0u : own ? OP_OWN_SYNC : 0xFFu;
+        for (int d = 1; d <= most; d++) {
+            const uint32_t q0 = __shfl_up_sync(0xffffffffu, r0, d), q1 = __shfl_up_sync(0xffffffffu, r1, d);
+            const uint32_t v0 = __shfl_up_sync(0xffffffffu, w0, d), v1 = __shfl_up_sync(0xffffffffu, w1, d);
+            if (simple && lane >= d && ((r0 <= v1 && v0 <= r1) || (w0 <= v1 && v0 <= w1) || (w0 <= q1 && q0 <= w1))) m |= 1u << (d - 1);
+        }
+        if (k0 > 0 && lane < OP_WINDOW && !own) m |= (0xFFu << lane) & 0x7Fu;
+        if (in) conf[k0 + lane] = (uint8_t)m;
+    }
+}
+
 // with_agents: the launch has 2 x npes CTAs, CTA npes + p being PE p's context agent
-__global__ void __launch_bounds__(INTERP_THREADS) k_interp(shmemg_device_ctx_t c, const shmemg_op_t *ops,
+__global__ void __launch_bounds__(INTERP_THREADS, 1) k_interp(shmemg_device_ctx_t c, const shmemg_op_t *ops,
                                                            int64_t nops, int64_t *fetched, int use_bulk,
                                                            int with_agents) {
     const int me = shmemg_d_my_pe(c);
@@ -450,6 +491,7 @@ __global__ void __launch_bounds__(INTERP_THREADS) k_interp(shmemg_device_ctx_t c
     // and the indices of the ops with a nonzero code, in order
     __shared__ uint8_t s_act[OP_BATCH];
     __shared__ uint8_t s_list[OP_BATCH];
+    __shared__ uint8_t s_conf[OP_BATCH];  // per listed op (op_conflicts)
     __shared__ int s_nact;
     // shared-team ops of a CTA-mode heap launched in clusters run inside the cluster: the
     // team barrier is the hardware cluster barrier, small alltoalls are staged in the
@@ -517,9 +559,15 @@ __global__ void __launch_bounds__(INTERP_THREADS) k_interp(shmemg_device_ctx_t c
         }
     };
     bool failed = false;
+    uint32_t rot = 0;
+    int q_sync = 0, nact_open = 0;  // listed ops q_sync .. nact_open - 1 have had no PE barrier after them yet
+    bool carry = false;             // ops of earlier batches neither
+    // granule of the conflict check: 16 bytes, or what makes the heap's count fit 32 bits
+    const int heap_bits = 64 - __clzll((long long)((uint64_t)c.npes * c.pe_stride)), gran = heap_bits > 36 ? heap_bits - 32 : 4;
     for (int64_t base = 0; base < nops && (!failed || dsm); base += OP_BATCH) {
     const int cnt = (int)(nops - base < OP_BATCH ? nops - base : OP_BATCH);
     if (mb && threadIdx.x == 0) *(volatile uint32_t *)&mb->beat = (uint32_t)(base / OP_BATCH) + 1;
+    carry |= q_sync < nact_open && c.pe_mode == SHMEMG_PE_MODE_CLUSTER;  // (a CTA's are, after this)
     __syncthreads();
     for (int q = threadIdx.x; q < cnt * 4; q += blockDim.x)
         reinterpret_cast<uint4 *>(s_ops)[q] = __ldcg(reinterpret_cast<const uint4 *>(ops + base) + q);
@@ -542,16 +590,28 @@ __global__ void __launch_bounds__(INTERP_THREADS) k_interp(shmemg_device_ctx_t c
             nact += __popc(m);
         }
         if (lane == 0) s_nact = nact;
+        __syncwarp();
+        op_conflicts(s_ops, s_act, s_list, s_conf, nact, c.pe_stride, gran);
     }
     __syncthreads();
     if (dma && dma_busy(s_dma)) dma_progress(s_dma, s_ring);  // background transfers advance
     const int nact = s_nact;
+    q_sync = 0;
+    nact_open = nact;
     // the PE's ops in order; once failed (only in a clustered CTA-mode launch) every
     // remaining op of the script, for its cluster barriers
     for (int qi = 0, k_next = 0;;) {
         int k;
         if (!failed) {
             if (qi >= nact) break;
+            const uint32_t conf = s_conf[qi];
+            const int open = qi - q_sync;
+            if ((open > 0 && (open > OP_WINDOW || (conf & ((1u << open) - 1u)))) || (carry && conf != OP_OWN_SYNC)) {
+                shmemg_d_pe_sync(c);
+                q_sync = qi;
+                carry = false;
+            }
+            if (conf & OP_APART) q_sync = qi + 1, carry = false;  // (begins or ends with a PE barrier, or completes at a quiet)
             k = s_list[qi++];
         } else {
             if (!dsm || k_next >= cnt) break;
@@ -561,7 +621,7 @@ __global__ void __launch_bounds__(INTERP_THREADS) k_interp(shmemg_device_ctx_t c
         const int64_t i = base + k;
         if (dma && dma_busy(s_dma)) dma_progress(s_dma, s_ring);  // background transfers advance
         const int act = s_act[k];
-        const shmemg_op_t o = s_ops[k];
+        const shmemg_op_t &o = s_ops[k];
         int rc = SHMEMG_SUCCESS;
         if (failed) {  // only in a clustered CTA-mode launch: walk on, through the barriers
             for (int b = cluster_barriers(o); b > 0; b--) shmemg_d_cluster_sync();
@@ -579,6 +639,16 @@ __global__ void __launch_bounds__(INTERP_THREADS) k_interp(shmemg_device_ctx_t c
         const bool active =
             !warp || (threadIdx.x < 32 && (c.pe_mode != SHMEMG_PE_MODE_CLUSTER || shmemg_d_cluster_ctarank() == 0));
         const shmemg_group gw = warp ? shmemg_d_group_warp() : g;
+        // small puts, gets and AMOs that follow each other start on different warps of the PE, so
+        // their latencies overlap
+        auto turn = [&](uint64_t bytes) {
+            shmemg_group t = g;
+            t.rank += rot;
+            if (t.rank >= t.size) t.rank -= t.size;
+            rot += bytes < 32 * 512 ? ((uint32_t)bytes / 512 + 1) * 32 : 0;  // the warps it occupies
+            while (rot >= t.size) rot -= t.size;
+            return t;
+        };
         if (staged(o)) {
             // the ring becomes this CTA's DSMEM window: no background chunk may still be in
             // it (every CTA of the cluster drains before the collective's entry barrier, so
@@ -589,52 +659,32 @@ __global__ void __launch_bounds__(INTERP_THREADS) k_interp(shmemg_device_ctx_t c
         switch (o.kind & SHMEMG_OP_KIND_MASK) {
         case SHMEMG_OP_PUT:
         case SHMEMG_OP_PUT_NBI:
-            if (o.issuer == me && o.kind == SHMEMG_OP_PUT_NBI && o.sub != 0 &&
-                ctx_aligned(c, shmemg_d_addr(c, o.pe, o.dst), shmemg_d_addr(c, me, o.src), o.n, use_bulk)) {
-                if (mb) {  // posted to the PE's agent
-                    if (threadIdx.x == 0)
-                        agent_post(c, mb, agent_epoch, ag_posted, o.sub, (uint64_t)shmemg_d_addr(c, o.pe, o.dst),
-                                   (uint64_t)shmemg_d_addr(c, me, o.src), o.n, i);
-                } else if (dma && ctx_home) {  // queued on its context, moved in the background
-                    dma_enqueue(c, s_dma, s_ring, o.sub, (uint64_t)shmemg_d_addr(c, o.pe, o.dst),
-                                (uint64_t)shmemg_d_addr(c, me, o.src), o.n, 0, 1);
-                }
-            } else if (o.issuer == me) {
-                if (warp) {
-                    if (active) shmemg_d_copy_group(gw, shmemg_d_addr(c, o.pe, o.dst), shmemg_d_addr(c, me, o.src), o.n);
-                } else {
-                    pe_copy(c, g, shmemg_d_addr(c, o.pe, o.dst), shmemg_d_addr(c, me, o.src), o.n, use_bulk, s_ring,
-                            s_dma, s_bars);
-                    if (o.kind == SHMEMG_OP_PUT) shmemg_d_pe_sync(c);
-                }
-            }
-            break;
         case SHMEMG_OP_GET:
         case SHMEMG_OP_GET_NBI:
-            if (o.issuer == me && o.kind == SHMEMG_OP_GET_NBI && o.sub != 0 &&
-                ctx_aligned(c, shmemg_d_addr(c, me, o.dst), shmemg_d_addr(c, o.pe, o.src), o.n, use_bulk)) {
-                if (mb) {
-                    if (threadIdx.x == 0)
-                        agent_post(c, mb, agent_epoch, ag_posted, o.sub, (uint64_t)shmemg_d_addr(c, me, o.dst),
-                                   (uint64_t)shmemg_d_addr(c, o.pe, o.src), o.n, i);
-                } else if (dma && ctx_home) {
-                    dma_enqueue(c, s_dma, s_ring, o.sub, (uint64_t)shmemg_d_addr(c, me, o.dst),
-                                (uint64_t)shmemg_d_addr(c, o.pe, o.src), o.n, 0, 1);
-                }
-            } else if (o.issuer == me) {
-                if (warp) {
-                    if (active) shmemg_d_copy_group(gw, shmemg_d_addr(c, me, o.dst), shmemg_d_addr(c, o.pe, o.src), o.n);
+            if (o.issuer == me) {
+                const uint32_t kind = o.kind & SHMEMG_OP_KIND_MASK;
+                const bool put = kind == SHMEMG_OP_PUT || kind == SHMEMG_OP_PUT_NBI;
+                uint8_t *const d = shmemg_d_addr(c, put ? o.pe : me, o.dst);
+                const uint8_t *const s = shmemg_d_addr(c, put ? me : o.pe, o.src);
+                if ((o.kind == SHMEMG_OP_PUT_NBI || o.kind == SHMEMG_OP_GET_NBI) && o.sub != 0 &&
+                    ctx_aligned(c, d, s, o.n, use_bulk)) {
+                    if (mb) {  // posted to the PE's agent
+                        if (threadIdx.x == 0)
+                            agent_post(c, mb, agent_epoch, ag_posted, o.sub, (uint64_t)d, (uint64_t)s, o.n, i);
+                    } else if (dma && ctx_home) {  // queued on its context, moved in the background
+                        dma_enqueue(c, s_dma, s_ring, o.sub, (uint64_t)d, (uint64_t)s, o.n, 0, 1);
+                    }
+                } else if (warp) {
+                    if (active) shmemg_d_copy_group(gw, d, s, o.n);
                 } else {
-                    pe_copy(c, g, shmemg_d_addr(c, me, o.dst), shmemg_d_addr(c, o.pe, o.src), o.n, use_bulk, s_ring,
-                            s_dma, s_bars);
-                    if (o.kind == SHMEMG_OP_GET) shmemg_d_pe_sync(c);
+                    pe_copy(c, turn(o.n), d, s, o.n, use_bulk, s_ring, s_dma, s_bars);
                 }
             }
             break;
         case SHMEMG_OP_FETCH_ADD:
         case SHMEMG_OP_COMPARE_SWAP:
         case SHMEMG_OP_FETCH_XOR:
-            if (o.issuer == me && leader) {
+            if (o.issuer == me && turn(8).rank == 0) {
                 int64_t old;
                 if (o.dtype == SHMEMG_INT64) {
                     int64_t *t = (int64_t *)shmemg_d_addr(c, o.pe, o.dst);
@@ -720,7 +770,9 @@ __global__ void __launch_bounds__(INTERP_THREADS) k_interp(shmemg_device_ctx_t c
             else if (active) rc = shmemg_d_alltoallmem_scoped(c, o.team, o.dst, o.src, o.n, i, cs, warp);
             break;
         case SHMEMG_OP_REDUCE:
-            if (active) rc = shmemg_d_reduce_scoped(c, o.team, o.dst, o.src, o.n, o.dtype, o.sub, i, cs, warp);
+            // (float trees 16 loads at a time: 32 would spill registers of the walk, which come
+            // back from L2 after every fence)
+            if (active) rc = shmemg_d_reduce_scoped<4>(c, o.team, o.dst, o.src, o.n, o.dtype, o.sub, i, cs, warp);
             break;
         default:
             if (leader) shmemg_d_set_status(c, SHMEMG_ERR_INVALID_ARG, i);

@@ -271,3 +271,70 @@ def test_reduce_float_extrema_of_special_values(sg, heapf, op, P):
         got = h.view(dst, p, torch.float32, n).cpu().numpy()
         assert np.array_equal(got.view(np.uint32), want.view(np.uint32))
     sg.team_destroy(team)
+
+
+@pytest.mark.parametrize("mode,cd", [(0, 1), (1, 2)])
+@pytest.mark.parametrize("span,biggest,seed", [(256, 64, 1), (4096, 3000, 2), (300000, 200000, 3)])
+def test_script_ops_of_one_pe_keep_their_order(sg, heapf, orc, mode, cd, span, biggest, seed):
+    """Puts, gets and AMOs of one PE over a few bytes, read after write, written after read and
+    twice written in every order: the result is the list's, whichever of them overlap in time."""
+    npes, H, nops = 3, (span + 4095) // 4096 * 4096 + 4096, 333
+    rng = np.random.RandomState(seed)
+    ops = np.zeros(nops, W.OP_DTYPE)
+    for i in range(nops):
+        o = ops[i]
+        o["issuer"], o["pe"] = 0, rng.randint(0, npes)
+        if rng.rand() < 0.3:
+            o["kind"], o["dtype"] = rng.choice([W.OP_FADD, W.OP_CSWAP, W.OP_FXOR]), W.DT_INT64
+            o["dst"], o["operand"], o["cond"] = 8 * rng.randint(0, span // 8), rng.randint(1, 1 << 40), 0
+            continue
+        n = int(np.exp(rng.rand() * np.log(biggest)))
+        if rng.rand() < 0.5:
+            n = max(16, n // 16 * 16)
+        a = 16 if n % 16 == 0 and rng.rand() < 0.7 else 1
+        o["kind"], o["n"] = rng.choice([W.OP_PUT, W.OP_GET]), n
+        o["dst"], o["src"] = rng.randint(0, (span - n) // a + 1) * a, rng.randint(0, (span - n) // a + 1) * a
+        if o["pe"] == 0 and o["dst"] < o["src"] + n and o["src"] < o["dst"] + n:
+            o["pe"] = 1                                   # (a copy onto itself is undefined)
+    h = heapf(npes, H, pe_mode=mode, cluster_dim=cd)
+    init = random_heap(npes, H, seed)
+    upload(h, init)
+    fetched = torch.zeros(nops, dtype=torch.int64, device="cuda")
+    sg.run_script(torch.from_numpy(ops.view(np.uint8).copy()).cuda(), nops, fetched)
+    torch.cuda.synchronize()
+    assert sg.get_status()[0] == 0
+    ref = orc.Heap(npes, H, init)
+    want = ref.run_script(ops)
+    assert first_diff(download(h), ref.mem) is None
+    amo = np.isin(ops["kind"], [W.OP_FADD, W.OP_CSWAP, W.OP_FXOR])
+    if want is not None:
+        assert np.array_equal(fetched.cpu().numpy()[amo], np.asarray(want)[amo])
+
+
+@pytest.mark.parametrize("npes", [1, 2, 5, 64])
+def test_barriers_back_to_back(sg, heapf, orc, npes):
+    """Consecutive barriers, in which PEs arrive at the next before the last has been folded:
+    every PE's word goes round the ring one place per barrier."""
+    rounds, H = 200, 8192
+    h = heapf(npes, H)
+    ops = []
+    for r in range(rounds):
+        for p in range(npes):
+            o = np.zeros(1, W.OP_DTYPE)[0]
+            o["kind"], o["issuer"], o["pe"], o["n"] = W.OP_PUT, p, (p + 1) % npes, 8
+            o["src"], o["dst"] = 16 * (r % 2), 16 * ((r + 1) % 2)
+            ops.append(o)
+        for _ in range(1 + r % 3):
+            o = np.zeros(1, W.OP_DTYPE)[0]
+            o["kind"], o["issuer"] = W.OP_BARRIER_ALL, -1
+            ops.append(o)
+    ops = np.array(ops, W.OP_DTYPE)
+    init = random_heap(npes, H, 5)
+    upload(h, init)
+    fetched = torch.zeros(len(ops), dtype=torch.int64, device="cuda")
+    sg.run_script(torch.from_numpy(ops.view(np.uint8).copy()).cuda(), len(ops), fetched)
+    torch.cuda.synchronize()
+    assert sg.get_status()[0] == 0
+    ref = orc.Heap(npes, H, init)
+    ref.run_script(ops)
+    assert first_diff(download(h), ref.mem) is None
