@@ -65,10 +65,23 @@ uint64_t balanced_grid(uint64_t nitems, uint64_t cap, int ngroups) {
 }
 
 int ctas_for(const void *kernel, int threads, size_t smem) {
+    struct Key {
+        const void *kernel;
+        size_t smem;
+        int threads, device;
+        bool operator==(const Key &o) const {
+            return kernel == o.kernel && smem == o.smem && threads == o.threads && device == o.device;
+        }
+    };
+    struct Hash {
+        size_t operator()(const Key &k) const {
+            return ((size_t)k.kernel >> 4) * 0x9E3779B97F4A7C15ull ^ (k.smem * 31 + (size_t)k.threads) * 0xC2B2AE3D27D4EB4Full ^
+                   (size_t)k.device;
+        }
+    };
     static std::mutex mu;
-    static std::unordered_map<std::string, int> cache;
-    char key[96];
-    snprintf(key, sizeof(key), "%p/%d/%zu/%d", kernel, threads, smem, g_state.device);
+    static std::unordered_map<Key, int, Hash> cache;
+    const Key key = {kernel, smem, threads, g_state.device};
     std::lock_guard<std::mutex> lk(mu);
     auto it = cache.find(key);
     if (it != cache.end()) return it->second;

@@ -195,22 +195,45 @@ def lib():
     return _lib
 
 
-def _call(name, *args):
+_fns = {}  # resolved entry points (a small call's kernel runs shorter than a lookup through lib())
+
+
+def _resolve(name):
     f = getattr(lib(), name, None)
     if f is None:
         raise RuntimeError(f"{name} is not exported by libshmemg")
-    rc = f(*args)
+    _fns[name] = f
+    return f
+
+
+def _call(name, *args):
+    rc = (_fns.get(name) or _resolve(name))(*args)
     if rc != SUCCESS:
         raise ShmemgError(rc, name)
     return rc
 
 
+def _first_stream():
+    """torch's current stream through the public call (which sets CUDA up); later calls ask
+    torch for the raw handle of the current device's stream where it offers that (0.3 us
+    instead of 3 for the Stream object)."""
+    global _current_stream
+    import torch
+
+    s = torch.cuda.current_stream().cuda_stream
+    raw, dev = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+    if raw is not None and dev is not None:
+        _current_stream = lambda: raw(dev())  # noqa: E731
+    return s
+
+
+_current_stream = _first_stream
+
+
 def _stream(s):
     """torch.cuda.Stream / int / None -> cudaStream_t as int."""
     if s is None:
-        import torch
-
-        return torch.cuda.current_stream().cuda_stream
+        return _current_stream()
     if isinstance(s, int):
         return s
     return s.cuda_stream
@@ -221,6 +244,8 @@ def _ptr(x):
         return None
     if isinstance(x, int):
         return x
+    if type(x) is Sym:
+        return x.ptr
     if hasattr(x, "ptr"):
         return x.ptr
     if hasattr(x, "data_ptr"):
