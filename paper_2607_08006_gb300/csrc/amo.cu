@@ -42,6 +42,7 @@ struct AmoArgs {
 constexpr int AMO_U = 2;  // atomics in flight per thread
 constexpr int AMO_PLAIN_CTAS = 3;
 __global__ void __launch_bounds__(AMO_THREADS, 6) k_amo_stream(AmoArgs a) {
+    stream_enter();
     __shared__ uint64_t s_val[AMO_THREADS];
     __shared__ uint64_t s_old[AMO_THREADS];
     const uint64_t nblk = (a.nops + AMO_THREADS - 1) / AMO_THREADS;
@@ -188,6 +189,7 @@ __device__ __forceinline__ unsigned long long *amo_addr(const AmoArgs &a, uint32
 }
 
 __global__ void __launch_bounds__(CB_THREADS, CB_MIN_BLOCKS) k_amo_combine(AmoArgs a) {
+    stream_enter();
     extern __shared__ __align__(16) unsigned char cb_smem[];
     unsigned long long *s_acc = (unsigned long long *)cb_smem;   // accumulator / counter, then the fetched base
     uint32_t *s_key = (uint32_t *)(s_acc + CB_SLOTS);            // (word << 2 | code) + 1, 0 = empty
@@ -456,12 +458,12 @@ int shmemg_amo_stream(int64_t *table, uint64_t words_per_pe, const uint32_t *ops
         }
         const uint64_t tiles = ((nops / S.npes + 1 + CB_TILE - 1) / CB_TILE) * S.npes;
         const int grid = (int)std::min<uint64_t>(tiles, (uint64_t)per_sm * S.sm_count);
-        k_amo_combine<<<grid, CB_THREADS, CB_SMEM, to_stream(stream)>>>(a);
+        launch_chained(k_amo_combine, grid, CB_THREADS, CB_SMEM, to_stream(stream), a);
     } else {
         const uint64_t ctas = (nops + AMO_THREADS - 1) / AMO_THREADS;
         const uint64_t cap = (flags & SHMEMG_AMO_AGGREGATE) ? (uint64_t)ctas_for((const void *)k_amo_stream, AMO_THREADS, 0)
                                                             : (uint64_t)AMO_PLAIN_CTAS * (uint64_t)S.sm_count;
-        k_amo_stream<<<(unsigned)std::min(ctas, cap), AMO_THREADS, 0, to_stream(stream)>>>(a);
+        launch_chained(k_amo_stream, (unsigned)std::min(ctas, cap), AMO_THREADS, 0, to_stream(stream), a);
     }
     return cuda_rc(cudaGetLastError());
 }

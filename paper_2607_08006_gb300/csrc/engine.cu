@@ -195,7 +195,7 @@ __device__ __forceinline__ void xfer_items(const Xfer &x) {
 
 // SHIFT: segments off the 16-byte boundaries; REP: stored to every team member
 template <bool SHIFT, bool REP>
-__global__ void __launch_bounds__(XFER_THREADS, 2) k_xfer(Xfer x) { xfer_items<SHIFT, REP>(x); }
+__global__ void __launch_bounds__(XFER_THREADS, 2) k_xfer(Xfer x) { stream_enter(); xfer_items<SHIFT, REP>(x); }
 
 // Broadcast / fcollect whose blocks lie off the 16-byte boundaries: a CTA puts a chunk of some
 // KiB together in shared memory and thread 0 bulk-stores it to every member -- one TMA store
@@ -207,6 +207,7 @@ __global__ void __launch_bounds__(XFER_THREADS, 2) k_xfer(Xfer x) { xfer_items<S
 // cause is not understood).
 constexpr uint32_t XS_SMEM = 3 * XFER_THREADS * XFER_U * 16;
 __global__ void __launch_bounds__(XFER_THREADS, 2) k_xfer_stage(Xfer x) {
+    stream_enter();
     extern __shared__ __align__(128) uint4 xs_stage[];
     const int base_pe = x.start + blockIdx.y * x.gstride;
     for (uint64_t item = blockIdx.x; item < x.nitems; item += gridDim.x) {
@@ -281,6 +282,7 @@ __device__ __forceinline__ XChunk xchunk(const Xfer &x, uint64_t item, int base_
 }
 
 __global__ void __launch_bounds__(32) k_xfer_bulk(Xfer x, uint8_t *state, uint64_t timeout_ns) {
+    stream_enter();
     extern __shared__ __align__(128) uint8_t ring[];
     __shared__ __align__(8) uint64_t bars[XB_STAGES];
     const int base_pe = x.start + blockIdx.y * x.gstride;
@@ -346,6 +348,7 @@ __global__ void __launch_bounds__(32) k_xfer_bulk(Xfer x, uint8_t *state, uint64
 // no count: the signal's release covers its threads' stores, ordered before it by the barrier)
 template <bool SHIFT>
 __global__ void __launch_bounds__(XFER_THREADS, 2) k_put_signal(Xfer x, uint64_t *sig, uint64_t val, int op, uint32_t *done) {
+    stream_enter();
     xfer_items<SHIFT, false>(x);
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -392,6 +395,7 @@ __device__ __forceinline__ void red_store(const Red &x, int pe0, int r0, int ste
 
 template <typename T, typename V, int OP>
 __global__ void __launch_bounds__(RED_THREADS) k_reduce(Red x) {
+    stream_enter();
     const int pe0 = x.start + blockIdx.y * x.gstride;
     for (uint64_t item = blockIdx.x; item < x.nitems; item += gridDim.x) {
         const uint64_t v0 = item * x.chunk_vec;
@@ -415,6 +419,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_reduce(Red x) {
 // any other is passed over, so a block other than the first starts at its first number.
 template <typename T, typename V, int OP, int G>
 __global__ void __launch_bounds__(RED_THREADS) k_reduce_split(Red x) {
+    stream_enter();
     constexpr int NL = sizeof(V) / sizeof(T);
     constexpr bool FLT = std::is_floating_point<T>::value;
     const int pe0 = x.start + blockIdx.y * x.gstride;
@@ -448,16 +453,16 @@ __global__ void __launch_bounds__(RED_THREADS) k_reduce_split(Red x) {
             if constexpr (FLT)
                 if (r0 < r1) acc = shmemg_tree_sum<V>(x.heap, x.H, pe0 + r0 * x.stride, x.stride, r1 - r0, off);
         } else if (r0 < r1) {
-            acc = member(r0, off);
-            int r = r0 + step;
-            for (; r + 7 * step < r1; r += 8 * step) {  // eight members' loads in flight
+            for (int r = r0; r < r1; r += 8 * step) {  // eight members' loads in flight, the last ones' too
                 V v[8];
 #pragma unroll
-                for (int u = 0; u < 8; u++) v[u] = member(r + u * step, off);
+                for (int u = 0; u < 8; u++)
+                    if (r + u * step < r1) v[u] = member(r + u * step, off);
+                if (r == r0) acc = v[0];
 #pragma unroll
-                for (int u = 0; u < 8; u++) comb(acc, v[u]);
+                for (int u = 0; u < 8; u++)
+                    if (r + u * step < r1 && r + u > r0) comb(acc, v[u]);
             }
-            for (; r < r1; r += step) comb(acc, member(r, off));
         }
         auto shuffle = [&](auto get) {
             V o;
@@ -519,6 +524,7 @@ __device__ __forceinline__ void rb_load(void *smem, const void *src, uint32_t by
 
 template <typename T, typename V, int OP>
 __global__ void __launch_bounds__(RB_THREADS, 1) k_reduce_bulk(Red x, uint8_t *state, uint64_t timeout_ns) {
+    stream_enter();
     extern __shared__ __align__(128) uint8_t rb[];
     __shared__ __align__(8) uint64_t bars[RB_MAX_STAGES];
     constexpr int NL = sizeof(V) / sizeof(T);
@@ -603,6 +609,7 @@ __global__ void __launch_bounds__(RB_THREADS, 1) k_reduce_bulk(Red x, uint8_t *s
 // ------------------------------------------------------------------ single-thread ops
 template <typename T>
 __global__ void k_amo(T *addr, int kind, T v, T cond, T *fetched) {
+    stream_enter();
     T old;
     if (kind == SHMEMG_OP_FETCH_ADD) old = atomicAdd(addr, v);
     else if (kind == SHMEMG_OP_COMPARE_SWAP) old = atomicCAS(addr, cond, v);
@@ -659,7 +666,7 @@ static int launch_xfer_stage(Xfer x, int ngroups, cudaStream_t s) {
     x.mgroups = member_groups(x, x.nitems, cap, ngroups);
     x.nitems *= (uint64_t)x.mgroups;
     dim3 grid((unsigned)(x.nitems < (1u << 30) ? x.nitems : 1u << 30), (unsigned)ngroups);
-    k_xfer_stage<<<grid, XFER_THREADS, XS_SMEM, s>>>(x);
+    launch_chained(k_xfer_stage, grid, XFER_THREADS, XS_SMEM, s, x);
     return cuda_rc(cudaGetLastError());
 }
 
@@ -698,9 +705,9 @@ static int launch_xfer_vec(Xfer x, int ngroups, cudaStream_t s, uint64_t *sig, u
     const uint64_t rounds = (x.nitems + per - 1) / per;
     const uint64_t gx = SHIFT || rep || sig ? balanced_grid(rounds, cap, ngroups) : rounds < (1u << 30) ? rounds : 1u << 30;
     dim3 grid((unsigned)gx, (unsigned)ngroups);
-    if (sig) k_put_signal<SHIFT><<<grid, block, 0, s>>>(x, sig, val, op, done);
-    else if (rep) k_xfer<SHIFT, true><<<grid, block, 0, s>>>(x);
-    else k_xfer<SHIFT, false><<<grid, block, 0, s>>>(x);
+    if (sig) launch_chained(k_put_signal<SHIFT>, grid, block, 0, s, x, sig, val, op, done);
+    else if (rep) launch_chained(k_xfer<SHIFT, true>, grid, block, 0, s, x);
+    else launch_chained(k_xfer<SHIFT, false>, grid, block, 0, s, x);
     return cuda_rc(cudaGetLastError());
 }
 
@@ -727,7 +734,7 @@ static int launch_xfer_bulk(Xfer x, int ngroups, cudaStream_t s) {
     x.mgroups = member_groups(x, x.nitems, cap, ngroups);
     x.nitems *= (uint64_t)x.mgroups;
     dim3 grid((unsigned)balanced_grid(x.nitems, cap, ngroups), (unsigned)ngroups);
-    k_xfer_bulk<<<grid, 32, XB_SMEM, s>>>(x, st().base, st().timeout_ns);
+    launch_chained(k_xfer_bulk, grid, 32, XB_SMEM, s, x, st().base, st().timeout_ns);
     return cuda_rc(cudaGetLastError());
 }
 
@@ -806,7 +813,7 @@ static int launch_red_v(Red r, int ngroups, cudaStream_t s) {
             const uint64_t C = r.rb_chunk, nchunks = (r.nvec * sizeof(V) + C - 1) / C;
             const uint64_t cap = (uint64_t)ctas_for((const void *)k_reduce_bulk<T, V, OP>, RB_THREADS, RB_SMEM);
             dim3 grid((unsigned)balanced_grid(nchunks, cap, ngroups), (unsigned)ngroups);
-            k_reduce_bulk<T, V, OP><<<grid, RB_THREADS, RB_SMEM, s>>>(r, st().base, st().timeout_ns);
+            launch_chained(k_reduce_bulk<T, V, OP>, grid, RB_THREADS, RB_SMEM, s, r, st().base, st().timeout_ns);
             return cuda_rc(cudaGetLastError());
         }
     }
@@ -822,8 +829,8 @@ static int launch_red_v(Red r, int ngroups, cudaStream_t s) {
             // form has a few hundred items its coalesced member loads win)
             if (r.nitems * (uint64_t)ngroups * 8 < cap) {
                 dim3 grid((unsigned)balanced_grid(ctas, cap, ngroups), (unsigned)ngroups);
-                if (G == 8) k_reduce_split<T, V, OP, 8><<<grid, RED_THREADS, 0, s>>>(r);
-                else k_reduce_split<T, V, OP, 4><<<grid, RED_THREADS, 0, s>>>(r);
+                if (G == 8) launch_chained(k_reduce_split<T, V, OP, 8>, grid, RED_THREADS, 0, s, r);
+                else launch_chained(k_reduce_split<T, V, OP, 4>, grid, RED_THREADS, 0, s, r);
                 return cuda_rc(cudaGetLastError());
             }
         }
@@ -843,7 +850,7 @@ static int launch_red_v(Red r, int ngroups, cudaStream_t s) {
         r.nitems = ones;
     }
     dim3 grid((unsigned)(queue ? r.nitems : balanced_grid(r.nitems, cap, ngroups)), (unsigned)ngroups);
-    k_reduce<T, V, OP><<<grid, RED_THREADS, 0, s>>>(r);
+    launch_chained(k_reduce<T, V, OP>, grid, RED_THREADS, 0, s, r);
     return cuda_rc(cudaGetLastError());
 }
 
@@ -882,7 +889,7 @@ static int amo(T *target, int kind, T v, T cond, int pe, T *fetched, void *strea
     if (sym_offset(target, sizeof(T), &off)) return SHMEMG_ERR_NOT_SYMMETRIC;
     if (off % sizeof(T)) return SHMEMG_ERR_INVALID_ARG;
     T *addr = (T *)(st().heap + (uint64_t)pe * st().H + off);
-    k_amo<T><<<1, 1, 0, to_stream(stream)>>>(addr, kind, v, cond, fetched);
+    launch_chained(k_amo<T>, 1, 1, 0, to_stream(stream), addr, kind, v, cond, fetched);
     return cuda_rc(cudaGetLastError());
 }
 

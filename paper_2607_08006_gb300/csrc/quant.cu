@@ -78,6 +78,7 @@ __device__ __forceinline__ void q_store(const QArgs &a, uint8_t *base, uint64_t 
 constexpr int Q_BLOCKS = 4;
 template <int FMT>
 __global__ void __launch_bounds__(Q_THREADS) k_quantize(QArgs a) {
+    stream_enter();
     const uint64_t nblk = (a.n + 127) / 128, ngrp = (nblk + Q_BLOCKS - 1) / Q_BLOCKS;
     const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x >> 5);
     const uint64_t wid = (uint64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -133,6 +134,7 @@ struct QSumArgs {
 // is accumulated).  The ragged tail runs in 4-element steps.
 template <int FMT, int E>
 __global__ void __launch_bounds__(Q_THREADS) k_qsum(QSumArgs a) {
+    stream_enter();
     constexpr int M = E == 4 ? 16 : 8;                         // members loaded ahead
     __shared__ __align__(128) float s_out[2][Q_THREADS * E];   // alternate chunk buffers
     const int pe0 = a.start + blockIdx.y * a.gstride;
@@ -163,7 +165,7 @@ static void launch_qsum_e(const QSumArgs &a, int ngroups, cudaStream_t s) {
     // us with resident CTAs taking chunks in turn, 115 so)
     const uint64_t gx = need * (uint64_t)ngroups <= 8 * cap ? need : balanced_grid(need, cap, ngroups);
     dim3 grid((unsigned)gx, (unsigned)ngroups);
-    k_qsum<FMT, E><<<grid, Q_THREADS, 0, s>>>(a);
+    launch_chained(k_qsum<FMT, E>, grid, Q_THREADS, 0, s, a);
 }
 template <int FMT>
 static void launch_qsum(const QSumArgs &a, int ngroups, cudaStream_t s) {
@@ -206,8 +208,8 @@ int shmemg_quantize(shmemg_team_t team, void *q, float *scales, const float *src
         const uint64_t warps = (nb + Q_BLOCKS - 1) / Q_BLOCKS * (uint64_t)t.size;
         const uint64_t ctas = (warps + (Q_THREADS / 32) - 1) / (Q_THREADS / 32);
         const unsigned grid = (unsigned)(ctas <= 64 * cap ? ctas : balanced_grid(ctas, cap));
-        if (e4) k_quantize<SHMEMG_FMT_E4M3><<<grid, Q_THREADS, 0, to_stream(stream)>>>(a);
-        else k_quantize<SHMEMG_FMT_BF16><<<grid, Q_THREADS, 0, to_stream(stream)>>>(a);
+        if (e4) launch_chained(k_quantize<SHMEMG_FMT_E4M3>, grid, Q_THREADS, 0, to_stream(stream), a);
+        else launch_chained(k_quantize<SHMEMG_FMT_BF16>, grid, Q_THREADS, 0, to_stream(stream), a);
     }
     return cuda_rc(cudaGetLastError());
 }

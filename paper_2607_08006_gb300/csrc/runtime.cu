@@ -460,11 +460,14 @@ const char *shmemg_strerror(int code) {
 }
 
 // --------------------------------------------------------------- ordering
-static __global__ void k_fence() { shmemg_d_fence_sys(); }
+static __global__ void k_fence() {
+    stream_enter();
+    shmemg_d_fence_sys();
+}
 
 int shmemg_fence(void *stream) {
     if (int rc = check_init()) return rc;
-    k_fence<<<1, 1, 0, to_stream(stream)>>>();
+    launch_chained(k_fence, 1, 1, 0, to_stream(stream));
     return cuda_rc(cudaGetLastError());
 }
 
@@ -484,7 +487,7 @@ int shmemg_team_sync(shmemg_team_t team, void *stream) {
     if (team_get(team, &t)) return SHMEMG_ERR_INVALID_ARG;
     // every member PE is driven by this host thread through `stream`: stream order is
     // the team barrier; enqueue a device fence so the barrier also orders memory
-    k_fence<<<1, 1, 0, to_stream(stream)>>>();
+    launch_chained(k_fence, 1, 1, 0, to_stream(stream));
     return cuda_rc(cudaGetLastError());
 }
 

@@ -1020,6 +1020,7 @@ __global__ void __launch_bounds__(SV_THREADS, 2) k_plain(SvArgs a, shmemg_req_t 
                                                       uint32_t nstage, int final, int status, PlainScratch *sc,
                                                       shmemg_completion_t *rec) {
     __shared__ unsigned long long s_amo;
+    stream_enter();
     if (lo == 0 && blockIdx.x == 0 && threadIdx.x == 0) sc->t_start = now_dev();
     uint64_t part = 0;
     if (status == SHMEMG_SUCCESS)
@@ -1260,11 +1261,10 @@ int shmemg_request_run(const shmemg_req_t *req, const shmemg_server_cfg_t *cfg_i
     SvArgs ka = a;
     const uint32_t ns = status == SHMEMG_SUCCESS ? g.nstage : 0;
     if (ns) {  // the staged payload first, then the operation
-        k_plain<<<grid_for(ns), SV_THREADS, 0, to_stream(stream)>>>(ka, *req, 0, ns, ns, 0, status, sc, rec);
+        launch_chained(k_plain, grid_for(ns), SV_THREADS, 0, to_stream(stream), ka, *req, 0u, ns, ns, 0, status, sc, rec);
         if (int rc = cuda_rc(cudaGetLastError())) return rc;
     }
-    k_plain<<<grid_for(g.ntiles - ns), SV_THREADS, 0, to_stream(stream)>>>(ka, *req, ns, g.ntiles, ns, 1, status, sc,
-                                                                           rec);
+    launch_chained(k_plain, grid_for(g.ntiles - ns), SV_THREADS, 0, to_stream(stream), ka, *req, ns, g.ntiles, ns, 1, status, sc, rec);
     return cuda_rc(cudaGetLastError());
 }
 
