@@ -6,7 +6,7 @@
 // Roles in the server kernel:
 //  * CTA 0, thread 0 -- the admitter: acquire-polls the ring tail in mapped host memory,
 //    validates the request, finds a free slot and its destination pages (one page range
-//    free on every PE the request writes: OR of the per-PE page bitmaps, first fit), marks
+//    free on every PE the request writes: OR of the per-PE page bitmaps, first fit), takes
 //    them, fills the slot and publishes (slot, generation) to the device work queue.
 //  * CTAs 1..W -- workers: take tiles of queued requests (a window of the queue's oldest
 //    entries, spread by CTA index so small requests run beside big ones), claim a tile by
@@ -31,7 +31,7 @@ constexpr int SRV_THREADS = SV_THREADS;
 constexpr uint64_t RMA_TILE = 64ull << 10;    // bytes per put/get tile
 constexpr uint64_t RED_TILE = 8192;           // elements per reduce tile
 constexpr uint64_t A2A_TILE = 32ull << 10;    // bytes per alltoall block chunk
-constexpr uint32_t WINDOW = 32;               // queue entries workers spread over
+constexpr uint32_t WINDOW = 32;               // queue entries workers spread over (a lane each)
 constexpr uint8_t FMT_F32 = 0xFF;
 
 struct SvHost {                      // mapped host memory
@@ -64,6 +64,10 @@ struct SvCtl {                       // device memory
     unsigned int sm_workers[SV_MAX_SMID];  // worker CTAs per SM id (each worker's rank on its SM)
 };
 
+// next tile of a slot without a request: above every tile count (geometry: under 2^30), and far
+// enough below 2^32 for the adds of late claimers
+constexpr unsigned long long CLAIM_NONE = 0x80000000ull;
+
 // One admitted request.  The claim word, which every worker that looks at the request
 // touches, has a cache line of its own; the completion count and checksum (one update
 // per published chunk) share another; the request fields are read-mostly.
@@ -93,7 +97,9 @@ struct SvArgs {
     int npes;
     shmemg_server_cfg_t cfg;
     uint32_t pages_per_pe, bm_words;
-    unsigned long long *bitmaps;     // npes * bm_words
+    unsigned long long *freed;       // npes * bm_words: pages given back since the admitter last looked
+    unsigned long long *shadow;      // the admitter's page bitmaps where they exceed SV_SHADOW_MAX, else null
+    int page_log2;                   // log2(cfg.page_bytes) when a power of two, else -1
     SvSlot *slots;
     uint32_t nslots;
     unsigned long long *fifo;        // (gen << 32) | slot
@@ -528,140 +534,198 @@ __device__ void write_completion(const SvArgs &a, uint64_t ticket, uint64_t t_ad
 }
 
 // ------------------------------------------------------------------ admitter
-// Page bitmaps, warp-collective (all 32 lanes call with the same arguments): lane m
-// handles members m, m + 32, ... of the request's PEs, so a request spread over P PEs
-// costs about P/32 dependent loads or atomics per bitmap word, not P.
-__device__ bool find_pages(const SvArgs &a, const Geo &g, uint32_t need, uint32_t *first, int lane) {
-    if (need == 0) { *first = 0; return true; }
-    if (need > a.pages_per_pe) return false;
+// The page bitmaps (a bit per page and PE, set = taken) belong to the admitter alone and live in
+// its shared memory while they fit: a request's pages are found and taken without leaving the
+// SM.  Workers give pages back by or-ing them into `freed` (release); the admitter collects a
+// PE's freed pages only when a request does not fit what it knows to be free.  Until it
+// does, a freed page counts as taken, which is safe.  (With the bitmaps in global memory, set by
+// the admitter and cleared by the workers, each request cost a chain of loads, a fence and
+// atomics: 3 us, and the admitter bound the engine.)
+constexpr size_t SV_SHADOW_MAX = 40u << 10;
+
+// First run of `need` clear bits in the OR of the members' bitmaps (all 32 lanes call with the
+// same arguments: lane m handles members m, m + 32, ...).
+__device__ bool find_run(const SvArgs &a, const unsigned long long *sh, const Geo &g, uint32_t need, uint32_t *first, int lane) {
     uint32_t run = 0;
     for (uint32_t w = 0; w < a.bm_words; w++) {
         unsigned long long mine = 0;
         for (int m = lane; m < g.count + g.count2; m += 32)
-            mine |= *(volatile unsigned long long *)&a.bitmaps[(uint64_t)geo_pe(g, m) * a.bm_words + w];
-        const unsigned long long occ = (unsigned long long)__reduce_or_sync(0xffffffffu, (unsigned)mine) |
-                                       ((unsigned long long)__reduce_or_sync(0xffffffffu, (unsigned)(mine >> 32)) << 32);
-        for (int b = 0; b < 64; b++) {
-            const uint32_t page = w * 64 + b;
-            if (page >= a.pages_per_pe) return false;
-            if ((occ >> b) & 1ull) {
-                run = 0;
-            } else if (++run == need) {
-                *first = page + 1 - need;
+            mine |= *(const volatile unsigned long long *)&sh[(uint64_t)geo_pe(g, m) * a.bm_words + w];
+        unsigned long long occ = (unsigned long long)__reduce_or_sync(0xffffffffu, (unsigned)mine) |
+                                 ((unsigned long long)__reduce_or_sync(0xffffffffu, (unsigned)(mine >> 32)) << 32);
+        const uint32_t left = a.pages_per_pe - w * 64;
+        if (left < 64) occ |= ~0ull << left;
+        for (uint32_t pos = 0; pos < 64;) {  // the word's runs of clear bits, then of set ones
+            const unsigned long long rest = occ >> pos;
+            const uint32_t z = rest ? (uint32_t)__ffsll((long long)rest) - 1 : 64 - pos;
+            if (run + z >= need) {
+                *first = w * 64 + pos - run;
                 return true;
             }
+            run += z;
+            pos += z;
+            if (pos >= 64) break;
+            run = 0;
+            const unsigned long long set = ~(occ >> pos);  // (the bits shifted in are set here)
+            pos += set ? (uint32_t)__ffsll((long long)set) - 1 : 64;
         }
     }
     return false;
 }
 
-__device__ void mark_pages(const SvArgs &a, const Geo &g, uint32_t p0, uint32_t np, bool set, int lane) {
-    for (int m = lane; m < g.count + g.count2; m += 32) {
-        unsigned long long *bm = a.bitmaps + (uint64_t)geo_pe(g, m) * a.bm_words;
-        for (uint32_t p = p0; p < p0 + np;) {
-            const uint32_t w = p / 64, b = p % 64;
-            const uint32_t nb = (64 - b) < (p0 + np - p) ? (64 - b) : (p0 + np - p);
-            const unsigned long long mask = (nb == 64 ? ~0ull : ((1ull << nb) - 1)) << b;
-            if (set) atomicOr(bm + w, mask);
-            else atomicAnd(bm + w, ~mask);
-            p += nb;
-        }
+__device__ __forceinline__ unsigned long long page_mask(uint32_t p, uint32_t end, uint32_t *nb) {
+    const uint32_t b = p % 64;
+    *nb = (64 - b) < (end - p) ? (64 - b) : (end - p);
+    return (*nb == 64 ? ~0ull : ((1ull << *nb) - 1)) << b;
+}
+
+// Finds and takes `need` pages at one range of every member; the members' freed pages are
+// collected only if the range is not found without them.
+__device__ bool take_pages(const SvArgs &a, unsigned long long *sh, const Geo &g, uint32_t need, uint32_t *first, int lane) {
+    *first = 0;
+    if (need == 0) return true;
+    if (!find_run(a, sh, g, need, first, lane)) {
+        bool got = false;
+        for (int m = lane; m < g.count + g.count2; m += 32)
+            for (uint32_t w = 0; w < a.bm_words; w++) {
+                const uint64_t at = (uint64_t)geo_pe(g, m) * a.bm_words + w;
+                if (*(volatile unsigned long long *)&a.freed[at] == 0) continue;
+                *(volatile unsigned long long *)&sh[at] = *(volatile unsigned long long *)&sh[at] & ~atomicExch(&a.freed[at], 0ull);
+                got = true;
+            }
+        if (!__any_sync(0xffffffffu, got)) return false;
+        shmemg_d_fence_gpu();  // the frees collected above happen before the pages' reuse
+        __syncwarp();
+        if (!find_run(a, sh, g, need, first, lane)) return false;
     }
+    for (int m = lane; m < g.count + g.count2; m += 32)
+        for (uint32_t p = *first, nb; p < *first + need; p += nb) {
+            const unsigned long long mask = page_mask(p, *first + need, &nb);
+            volatile unsigned long long *w = &sh[(uint64_t)geo_pe(g, m) * a.bm_words + p / 64];
+            *w = *w | mask;
+        }
+    __syncwarp();
+    return true;
+}
+
+// A finished request's pages back to the admitter (the finalizing warp)
+__device__ void give_pages(const SvArgs &a, const Geo &g, uint32_t p0, uint32_t np, int lane) {
+    shmemg_d_fence_gpu();  // the tiles' reads and writes happen before the pages' reuse
+    for (int m = lane; m < g.count + g.count2; m += 32)
+        for (uint32_t p = p0, nb; p < p0 + np; p += nb) {
+            const unsigned long long mask = page_mask(p, p0 + np, &nb);
+            atomicOr(a.freed + (uint64_t)geo_pe(g, m) * a.bm_words + p / 64, mask);
+        }
     __syncwarp();
 }
 
-// Admission state of the admitter (lane 0 of CTA 0's first warp).
+// Admission state of the admitter warp (the same in every lane but slot_gen).
+constexpr int PUB = 8;  // admitted requests published together
 struct AdmState {
-    uint64_t fifo_tail, fifo_published;
-    uint32_t rot;
+    uint64_t fifo_tail, fifo_head;   // entries written; the last known head
+    uint32_t win, slot_free;         // slots win .. win + 31 (mod nslots): those seen free
+    uint32_t slot_gen;               // lane i: slot win + i's generation
+    int npub;                        // admitted, unpublished requests
 };
 
-// Publishes the slots admitted since the last flush: one GPU-scope fence orders every
-// slot field and claim word before the queue tail that workers acquire.
-__device__ __forceinline__ void adm_flush(const SvArgs &a, AdmState &st) {
-    if (st.fifo_published == st.fifo_tail) return;
+// Publishes the slots admitted since the last flush: one GPU-scope fence orders every slot
+// field before the claim words, another the claim words and entries before the queue tail
+// that workers acquire.  s_pub: their (gen, slot) entries.
+__device__ __forceinline__ void adm_flush(const SvArgs &a, AdmState &st, const unsigned long long *s_pub, int lane) {
+    if (st.npub == 0) return;
+    __syncwarp();
+    const unsigned long long e = lane < st.npub ? s_pub[lane] : 0ull;
+    SvSlot &s = a.slots[(uint32_t)e];
+    if (lane < st.npub) s.t_pub = now_dev();
+    if (lane == 0) atomicAdd(&a.ctl->inflight, (unsigned long long)st.npub);
     shmemg_d_fence_gpu();
-    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(&a.ctl->fifo_tail), "l"((unsigned long long)st.fifo_tail)
-                 : "memory");
-    st.fifo_published = st.fifo_tail;
+    __syncwarp();
+    if (lane < st.npub) {
+        // a worker whose fetch-and-add sees this generation also sees the slot's fields
+        *(volatile unsigned long long *)&s.claim = e & 0xFFFFFFFF00000000ull;
+        a.fifo[(st.fifo_tail - st.npub + lane) % a.fifo_cap] = e;
+    }
+    __syncwarp();
+    if (lane == 0)
+        asm volatile("fence.acq_rel.gpu;\n\tst.release.gpu.global.u64 [%0], %1;" ::"l"(&a.ctl->fifo_tail),
+                     "l"((unsigned long long)st.fifo_tail)
+                     : "memory");
+    __syncwarp();
+    st.npub = 0;
 }
 
-// Tries to admit one request: 1 = admitted (or completed with an error), 0 = no slot,
-// queue room or pages yet (retry later).  Warp-collective: every lane computes the same
-// verdict (lane 0's reads are broadcast); lane 0 writes the slot and the queue.
-__device__ int adm_try(const SvArgs &a, AdmState &st, const shmemg_req_t &r, uint64_t now, int lane) {
+// Tries to admit one request (in shared memory): 1 = admitted (or completed with an error), 0 =
+// no slot, queue room or pages yet (retry later).  Warp-collective: every lane computes the
+// same verdict.
+__device__ int adm_try(const SvArgs &a, AdmState &st, unsigned long long *sh, unsigned long long *s_pub, const shmemg_req_t &r,
+                       uint64_t now, int lane) {
     const Geo g = geometry(r, a.npes, a.H, a.cfg.amo_words);
     if (!g.valid) {
         if (lane == 0) write_completion(a, r.ticket, now, 0, SHMEMG_ERR_INVALID_ARG);
         __syncwarp();
         return 1;
     }
-    const uint32_t need = (uint32_t)((g.bytes + a.cfg.page_bytes - 1) / a.cfg.page_bytes);
-    if (need > a.pages_per_pe) {
+    const uint64_t up = g.bytes + a.cfg.page_bytes - 1;
+    const uint64_t pages = a.page_log2 >= 0 ? up >> a.page_log2 : up / a.cfg.page_bytes;
+    if (pages > a.pages_per_pe) {
         if (lane == 0) write_completion(a, r.ticket, now, 0, SHMEMG_ERR_OUT_OF_HEAP);
         __syncwarp();
         return 1;
     }
-    int slot = -1;
-    if (lane == 0) {
-        // the queue head and the first candidate slot are read together; a slot is taken
-        // only through an acquire load of its busy word (its finalizer released it)
-        const uint32_t k0 = st.rot % a.nslots;
-        const unsigned long long head = *(volatile unsigned long long *)&a.ctl->fifo_head;
-        const uint32_t b0 = shmemg_d_ld_acquire_u32(&a.slots[k0].busy);
-        if (st.fifo_tail - head < a.fifo_cap) {
-            if (b0 == 0) slot = (int)k0;
-            for (uint32_t i = 1; i < a.nslots && slot < 0; i++) {
-                const uint32_t k = (st.rot + i) % a.nslots;
-                if (shmemg_d_ld_acquire_u32(&a.slots[k].busy) == 0) slot = (int)k;
-            }
-        }
+    const uint32_t need = (uint32_t)pages;
+    // queue room, by the last known head first
+    if (st.fifo_tail - st.fifo_head >= a.fifo_cap) {
+        st.fifo_head = *(volatile unsigned long long *)&a.ctl->fifo_head;
+        st.fifo_head = __shfl_sync(0xffffffffu, st.fifo_head, 0);
+        if (st.fifo_tail - st.fifo_head >= a.fifo_cap) return 0;
     }
-    slot = __shfl_sync(0xffffffffu, slot, 0);
-    if (slot < 0) return 0;
+    // a free slot: 32 are looked at together, through acquire loads of their busy words (their
+    // finalizers released them), and used up before the next 32
+    for (uint32_t seen = 0; st.slot_free == 0; seen += 32) {
+        if (seen >= a.nslots + 32) return 0;
+        __syncwarp();  // (slots taken just before are busy to these loads)
+        st.win = st.win + 32 < a.nslots ? st.win + 32 : 0;
+        const uint32_t k = st.win + (uint32_t)lane;
+        bool ok = k < a.nslots;
+        if (ok) {
+            st.slot_gen = *(volatile uint32_t *)&a.slots[k].gen;
+            ok = shmemg_d_ld_acquire_u32(&a.slots[k].busy) == 0;
+        }
+        st.slot_free = __ballot_sync(0xffffffffu, ok);
+    }
     uint32_t p0 = 0;
-    if (!find_pages(a, g, need, &p0, lane)) return 0;
-    if (need) shmemg_d_fence_gpu();  // page frees seen above happen before the pages' reuse
-    mark_pages(a, g, p0, need, true, lane);
+    if (!take_pages(a, sh, g, need, &p0, lane)) return 0;
+    const int j = __ffs((int)st.slot_free) - 1;
+    st.slot_free &= st.slot_free - 1;
+    const uint32_t slot = st.win + (uint32_t)j, gen = __shfl_sync(0xffffffffu, st.slot_gen, j) + 1;
     SvSlot &s = a.slots[slot];
-    if (lane == 0) {
-        const uint32_t gen = s.gen + 1;
-        s.req = r;
+    if (lane < 4) reinterpret_cast<uint4 *>(&s.req)[lane] = reinterpret_cast<const uint4 *>(&r)[lane];
+    if (lane == 4) {
         s.dst_off = a.cfg.arena_offset + (uint64_t)p0 * a.cfg.page_bytes;
         s.page0 = p0;
         s.npages = need;
         s.ntiles = g.ntiles;
-        s.nstage = g.nstage;
-        s.staged = 0;
         s.gen = gen;
-        s.done = 0;
-        s.checksum = 0;
         s.t_admit = now;
         s.status = 0;
         s.busy = 1;
-        // release: a worker whose fetch-and-add sees this generation also sees the fields
-        // above (and the page marks, ordered before it by the warp barrier)
-        asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(&s.claim), "l"((unsigned long long)gen << 32)
-                     : "memory");
-        atomicAdd(&a.ctl->inflight, 1ull);
-        a.fifo[st.fifo_tail % a.fifo_cap] = ((unsigned long long)gen << 32) | (unsigned)slot;
-        s.t_pub = now_dev();
+        s.nstage = g.nstage;
+        s.done = 0;
+        s.staged = 0;
+        s.checksum = 0;
+        s_pub[st.npub] = ((unsigned long long)gen << 32) | slot;
     }
-    __syncwarp();
     st.fifo_tail++;
-    st.rot = (uint32_t)slot + 1;
+    if (++st.npub == PUB) adm_flush(a, st, s_pub, lane);
     return 1;
 }
 
-// The admitter warp: each round it acquires the ring tail, reads up to 8 requests with
-// one 16-byte system-scope load per lane (4 lanes per 64-byte request), admits them in
-// order on lane 0 and publishes the batch with one fence.
 // The admitter warp keeps up to PEND requests taken from the ring and admits any of
 // them that fits now (oldest first), so a request waiting for pages does not hold back
 // later ones; once the oldest has waited AGE_NS, only it is tried until it is admitted
-// (no starvation).  Each round the warp acquires the ring tail and reads up to 8 new
-// requests with one 16-byte system-scope load per lane (4 lanes per 64-byte request);
-// admitted requests are published with one fence per round.
+// (no starvation).  Each round the warp acquires the ring tail and reads as many new
+// requests as it has room for with 16-byte system-scope loads (4 lanes per 64-byte
+// request, up to four per lane in flight); admitted requests are published PUB at a time.
 constexpr int PEND = 32;
 constexpr uint64_t AGE_NS = 2000000;
 
@@ -671,8 +735,12 @@ __device__ void admitter_warp(const SvArgs &a) {
     __shared__ int s_ctl[2];
     __shared__ int s_npend, s_adm;
     const int lane = threadIdx.x & 31;
+    __shared__ unsigned long long s_pub[PUB];
+    extern __shared__ unsigned long long sv_shadow[];
+    unsigned long long *sh = a.shadow ? a.shadow : sv_shadow;
+    for (uint32_t k = lane; k < (uint32_t)a.npes * a.bm_words; k += 32) sh[k] = 0ull;
     uint64_t head = 0;
-    AdmState st = {0, 0, 0};
+    AdmState st = {0, 0, a.nslots, 0, 0, 0};
     const uint64_t t_start = now_dev();
     uint64_t t_last = t_start;
     uint32_t sleep_ns = 64;
@@ -682,7 +750,7 @@ __device__ void admitter_warp(const SvArgs &a) {
         if (lane == 0) {
             const uint64_t now = now_dev();
             const uint64_t tail = shmemg_d_ld_acquire_sys_u64(&a.host->tail);
-            const uint64_t room = (uint64_t)(PEND - s_npend) < 8 ? (uint64_t)(PEND - s_npend) : 8;
+            const uint64_t room = (uint64_t)(PEND - s_npend);
             int nnew = (int)(tail - head < room ? tail - head : room), stop = 0;
             if (now - t_start > a.cfg.max_ns) stop = 1;
             if (nnew == 0 && s_npend == 0 && !stop) {
@@ -697,15 +765,19 @@ __device__ void admitter_warp(const SvArgs &a) {
         if (s_ctl[1]) break;
         if (nnew > 0) {
             const int q = lane >> 2, part = lane & 3, base = s_npend;
-            if (q < nnew) {
-                const uint32_t *p = (const uint32_t *)(a.ring + ((head + q) % a.ring_slots)) + 4 * part;
-                uint4 v;
-                asm volatile("ld.relaxed.sys.global.v4.u32 {%0, %1, %2, %3}, [%4];"
-                             : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-                             : "l"(p)
-                             : "memory");
-                reinterpret_cast<uint4 *>(&s_pend[base + q])[part] = v;
-            }
+            uint4 v[PEND / 8];
+#pragma unroll
+            for (int i = 0; i < PEND / 8; i++)
+                if (q + 8 * i < nnew) {
+                    const uint32_t *p = (const uint32_t *)(a.ring + ((head + q + 8 * i) % a.ring_slots)) + 4 * part;
+                    asm volatile("ld.relaxed.sys.global.v4.u32 {%0, %1, %2, %3}, [%4];"
+                                 : "=r"(v[i].x), "=r"(v[i].y), "=r"(v[i].z), "=r"(v[i].w)
+                                 : "l"(p)
+                                 : "memory");
+                }
+#pragma unroll
+            for (int i = 0; i < PEND / 8; i++)
+                if (q + 8 * i < nnew) reinterpret_cast<uint4 *>(&s_pend[base + q + 8 * i])[part] = v[i];
             head += (uint64_t)nnew;  // every lane: the next read uses it
         }
         __syncwarp();
@@ -720,7 +792,7 @@ __device__ void admitter_warp(const SvArgs &a) {
             int k = 0;
             for (int i = 0; i < n; i++) {  // the whole warp admits, in order
                 const bool try_it = !aged || i == 0;
-                if (try_it && adm_try(a, st, s_pend[i], now, lane)) {
+                if (try_it && adm_try(a, st, sh, s_pub, s_pend[i], now, lane)) {
                     admitted++;
                     continue;
                 }
@@ -734,9 +806,9 @@ __device__ void admitter_warp(const SvArgs &a) {
             if (lane == 0) s_npend = k;
             __syncwarp();
         }
+        adm_flush(a, st, s_pub, lane);
         if (lane == 0) {
             const uint64_t now = now_dev();
-            adm_flush(a, st);
             if (nnew > 0)
                 asm volatile("st.release.sys.global.u64 [%0], %1;" ::"l"((const uint64_t *)&a.host->head), "l"(head)
                              : "memory");
@@ -762,12 +834,15 @@ __device__ void admitter_warp(const SvArgs &a) {
 __device__ void finalize(const SvArgs &a, SvSlot &s, int lane) {
     const shmemg_req_t r = s.req;
     const Geo g = geometry(r, a.npes, a.H, a.cfg.amo_words);
-    if (s.npages) mark_pages(a, g, s.page0, s.npages, false, lane);
+    if (lane == 0) write_completion(a, r.ticket, s.t_admit, s.checksum, s.status);
+    __syncwarp();
+    if (s.npages) give_pages(a, g, s.page0, s.npages, lane);
     if (lane == 0) {
-        write_completion(a, r.ticket, s.t_admit, s.checksum, s.status);
+        // no look at the slot finds a tile left, whatever tile count the admitter writes next,
+        // until it publishes the next claim word
+        *(volatile unsigned long long *)&s.claim = ((unsigned long long)s.gen << 32) | CLAIM_NONE;
         atomicAdd(&a.ctl->inflight, ~0ull);  // -1
-        // the release orders the page frees (warp barrier above) and the count before the
-        // slot's reuse
+        // the release orders the count, and this warp's reads of the slot, before its reuse
         asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(&s.busy), "r"(0u) : "memory");
     }
     __syncwarp();
@@ -857,13 +932,14 @@ __device__ void worker(const SvArgs &a) {
     __shared__ uint64_t s_dst;
     __shared__ uint32_t s_nstage;
     const uint32_t me = blockIdx.x - 1;
-    bool primary = true;
+    bool primary = true;  // (warp 0)
     if (threadIdx.x == 0) s_fin = -1;
     if (threadIdx.x == 0) {
         uint32_t smid;
         asm volatile("mov.u32 %0, %%smid;" : "=r"(smid));
         primary = atomicAdd(&a.ctl->sm_workers[smid % SV_MAX_SMID], 1u) == 0;
     }
+    if (threadIdx.x < 32) primary = __shfl_sync(0xffffffffu, (int)primary, 0) != 0;
     const uint32_t max_sleep = primary ? 256 : 1024;
     unsigned long long idle_tail = ~0ull;  // thread 0: queue tail of the last scan that found it empty
     uint32_t sleep_ns = 32;
@@ -872,55 +948,86 @@ __device__ void worker(const SvArgs &a) {
     uint64_t pend_sum = 0;
     unsigned long long pend_amo = 0;
     for (;;) {
-        if (threadIdx.x == 0) {
+        if (threadIdx.x < 32) {
+            const int lane = (int)threadIdx.x;
             int cmd = 0;
-            uint32_t tile, cnt;
-            if (sticky >= 0 && claim_tiles(a, (uint32_t)sticky, &tile, &cnt, &s_req, &s_dst, &s_nstage)) {
-                s_slot = (uint32_t)sticky;
-                s_tile = tile;
-                s_cnt = cnt;
-                cmd = 1;
-            } else {
-                if (pend_cnt && publish(a, (uint32_t)sticky, pend_sum, pend_amo, pend_cnt))  // leaving the slot
-                    s_fin = sticky;
-                pend_cnt = 0;
-                pend_sum = 0;
-                sticky = -1;
+            if (lane == 0) {
+                uint32_t tile, cnt;
+                if (sticky >= 0 && claim_tiles(a, (uint32_t)sticky, &tile, &cnt, &s_req, &s_dst, &s_nstage)) {
+                    s_slot = (uint32_t)sticky;
+                    s_tile = tile;
+                    s_cnt = cnt;
+                    cmd = 1;
+                } else {
+                    if (pend_cnt && publish(a, (uint32_t)sticky, pend_sum, pend_amo, pend_cnt))  // leaving the slot
+                        s_fin = sticky;
+                    pend_cnt = 0;
+                    pend_sum = 0;
+                    sticky = -1;
+                }
             }
+            cmd = __shfl_sync(0xffffffffu, cmd, 0);
+            // The warp looks at the queue's WINDOW oldest entries at once (an entry costs two
+            // dependent trips to L2, one lane each): the leading exhausted ones leave the queue
+            // together, and the worker claims from the first one with tiles at or after its own
+            // place.  (One thread looked at one entry after the other and the head moved one entry a
+            // trip: two microseconds a one-tile request, whatever the number of workers.)
             for (int tries = 0; tries < 64 && cmd == 0; tries++) {
-                if (*(volatile unsigned int *)&a.ctl->exit_flag) { cmd = -1; break; }
-                if (idle_tail != ~0ull && *(volatile unsigned long long *)&a.ctl->fifo_tail == idle_tail) break;
-                const unsigned long long h = shmemg_d_ld_acquire_u64((const uint64_t *)&a.ctl->fifo_head);
-                const unsigned long long t = shmemg_d_ld_acquire_u64((const uint64_t *)&a.ctl->fifo_tail);
-                if (h >= t) {
-                    idle_tail = t;  // nothing queued: nothing new until the tail moves
+                unsigned long long h = 0, t = 0;
+                int go = 1;  // 1 look, 0 nothing new, -1 leave
+                if (lane == 0) {
+                    if (*(volatile unsigned int *)&a.ctl->exit_flag) go = -1;
+                    else if (idle_tail != ~0ull && *(volatile unsigned long long *)&a.ctl->fifo_tail == idle_tail) go = 0;
+                    else {
+                        h = shmemg_d_ld_acquire_u64((const uint64_t *)&a.ctl->fifo_head);
+                        t = shmemg_d_ld_acquire_u64((const uint64_t *)&a.ctl->fifo_tail);
+                        if (h >= t) {
+                            idle_tail = t;  // nothing queued: nothing new until the tail moves
+                            go = 0;
+                        } else {
+                            idle_tail = ~0ull;
+                        }
+                    }
+                }
+                go = __shfl_sync(0xffffffffu, go, 0);
+                if (go <= 0) {
+                    cmd = go;
                     break;
                 }
-                idle_tail = ~0ull;
+                h = __shfl_sync(0xffffffffu, h, 0);  // (orders the other lanes' reads after the acquires)
+                t = __shfl_sync(0xffffffffu, t, 0);
                 const uint32_t live = (uint32_t)((t - h) < WINDOW ? (t - h) : WINDOW);
-                const uint32_t start = me % live;
-                for (uint32_t j = 0; j < live && cmd == 0; j++) {
-                    const unsigned long long pos = h + (start + j) % live;
-                    const unsigned long long e = *(volatile unsigned long long *)&a.fifo[pos % a.fifo_cap];
-                    const uint32_t slot = (uint32_t)e, gen = (uint32_t)(e >> 32);
-                    SvSlot &s = a.slots[slot];
-                    const unsigned long long c = *(volatile unsigned long long *)&s.claim;
-                    const uint32_t nt = *(volatile uint32_t *)&s.ntiles;
-                    if ((uint32_t)(c >> 32) != gen || (uint32_t)c >= nt) {
-                        if (pos == h) atomicCAS(&a.ctl->fifo_head, h, h + 1);  // exhausted or stale head
-                        continue;
+                const bool valid = (uint32_t)lane < live;
+                const unsigned long long e = valid ? *(volatile unsigned long long *)&a.fifo[(h + lane) % a.fifo_cap] : 0ull;
+                SvSlot &q = a.slots[(uint32_t)e];
+                const unsigned long long c = *(volatile unsigned long long *)&q.claim;
+                const uint32_t nt = *(volatile uint32_t *)&q.ntiles;
+                const uint64_t t_pub = *(volatile uint64_t *)&q.t_pub;
+                const bool dead = (uint32_t)(c >> 32) != (uint32_t)(e >> 32) || (uint32_t)c >= nt;  // exhausted, or of a reused slot
+                const unsigned gone = __ballot_sync(0xffffffffu, valid && dead);
+                unsigned ready = __ballot_sync(0xffffffffu, valid && !dead && (primary || now_dev() - t_pub >= SECONDARY_DELAY_NS));
+                const int lead = __ffs((int)~gone) - 1;  // (-1: all 32)
+                if (lane == 0 && lead != 0) atomicCAS(&a.ctl->fifo_head, h, h + (lead < 0 ? 32 : lead));
+                while (ready && cmd == 0) {
+                    const unsigned from = ready & (~0u << (me % live));
+                    const int pick = __ffs((int)(from ? from : ready)) - 1;
+                    const uint32_t slot = __shfl_sync(0xffffffffu, (uint32_t)e, pick), ntp = __shfl_sync(0xffffffffu, nt, pick);
+                    if (lane == 0) {
+                        uint32_t tile, cnt;
+                        if (claim_tiles(a, slot, &tile, &cnt, &s_req, &s_dst, &s_nstage, ntp)) {  // (looked at just above)
+                            s_slot = slot;
+                            s_tile = tile;
+                            s_cnt = cnt;
+                            sticky = (int)slot;
+                            cmd = 1;
+                        }
                     }
-                    if (!primary && now_dev() - *(volatile uint64_t *)&s.t_pub < SECONDARY_DELAY_NS) continue;
-                    if (claim_tiles(a, slot, &tile, &cnt, &s_req, &s_dst, &s_nstage, nt)) {   // claim word and tile count read just above
-                        s_slot = slot;
-                        s_tile = tile;
-                        s_cnt = cnt;
-                        sticky = (int)slot;
-                        cmd = 1;
-                    }
+                    cmd = __shfl_sync(0xffffffffu, cmd, 0);
+                    ready &= ~(1u << pick);
                 }
             }
-            s_cmd = cmd;
+            if (lane == 0)
+                s_cmd = cmd;
         }
         __syncthreads();
         if (s_fin >= 0) {  // warp 0 finalizes the request this CTA completed
@@ -1131,7 +1238,10 @@ int shmemg_server_start(const shmemg_server_cfg_t *cfg_in, void *stream, shmemg_
     size_t off_slots = (bm_bytes + 255) & ~(size_t)255;
     size_t off_fifo = off_slots + (((size_t)a.nslots * sizeof(SvSlot) + 255) & ~(size_t)255);
     size_t off_ctl = off_fifo + (((size_t)a.fifo_cap * 8 + 255) & ~(size_t)255);
-    size_t total = off_ctl + sizeof(SvCtl);
+    const bool shadow_smem = bm_bytes <= SV_SHADOW_MAX;
+    const size_t smem = shadow_smem ? bm_bytes : 0;
+    size_t off_shadow = (off_ctl + sizeof(SvCtl) + 255) & ~(size_t)255;
+    size_t total = off_shadow + (shadow_smem ? 0 : bm_bytes);
     int rc = cuda_rc(cudaMalloc(&s->dev_mem, total));
     if (!rc) rc = cuda_rc(cudaMemset(s->dev_mem, 0, total));
     if (!rc) rc = cuda_rc(cudaHostAlloc((void **)&s->host, sizeof(SvHost), cudaHostAllocMapped));
@@ -1142,7 +1252,9 @@ int shmemg_server_start(const shmemg_server_cfg_t *cfg_in, void *stream, shmemg_
     memset(s->ring, 0, sizeof(shmemg_req_t) * a.ring_slots);
     memset(s->comp, 0, sizeof(shmemg_completion_t) * a.ring_slots);
     uint8_t *d = (uint8_t *)s->dev_mem;
-    a.bitmaps = (unsigned long long *)d;
+    a.freed = (unsigned long long *)d;
+    a.shadow = shadow_smem ? nullptr : (unsigned long long *)(d + off_shadow);
+    a.page_log2 = (cfg.page_bytes & (cfg.page_bytes - 1)) ? -1 : __builtin_ctzll(cfg.page_bytes);
     a.slots = (SvSlot *)(d + off_slots);
     a.fifo = (unsigned long long *)(d + off_fifo);
     a.ctl = (SvCtl *)(d + off_ctl);
@@ -1154,7 +1266,7 @@ int shmemg_server_start(const shmemg_server_cfg_t *cfg_in, void *stream, shmemg_
     if ((rc = cuda_rc(cudaHostGetDevicePointer(&p, s->comp, 0)))) { server_free(s); return rc; }
     a.comp = (shmemg_completion_t *)p;
     int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_server, SRV_THREADS, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_server, SRV_THREADS, smem);
     int cap = per_sm * S.sm_count;
     int workers = cfg.workers > 0 ? cfg.workers : cap - 1;
     if (workers < 1 || workers + 1 > cap) { server_free(s); return SHMEMG_ERR_UNSUPPORTED; }
@@ -1162,6 +1274,7 @@ int shmemg_server_start(const shmemg_server_cfg_t *cfg_in, void *stream, shmemg_
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3(workers + 1);
     lc.blockDim = dim3(SRV_THREADS);
+    lc.dynamicSmemBytes = smem;
     lc.stream = s->stream;
     cudaLaunchAttribute at;
     at.id = cudaLaunchAttributeCooperative;
@@ -1233,7 +1346,7 @@ int shmemg_server_stop(shmemg_server_t s) {
         if (e == cudaSuccess) break;
         if (e != cudaErrorNotReady) { rc = cuda_rc(e); break; }
         if (host_ns() > give_up) return SHMEMG_ERR_TIMEOUT;  // kernel still running: keep its memory
-        std::this_thread::sleep_for(std::chrono::microseconds(200));
+        std::this_thread::sleep_for(std::chrono::microseconds(20));
     }
     server_free(s);
     return rc;

@@ -338,3 +338,62 @@ def test_barriers_back_to_back(sg, heapf, orc, npes):
     ref = orc.Heap(npes, H, init)
     ref.run_script(ops)
     assert first_diff(download(h), ref.mem) is None
+
+
+@pytest.mark.parametrize("npes,arena_pages,inflight,count", [(4, 3, 1, 60), (8, 70, 5, 400), (33, 130, 64, 1000), (90, 4096, 1024, 1500)])
+def test_serving_page_and_slot_reuse(sg, heapf, npes, arena_pages, inflight, count):
+    """Few slots and pages reused many times, runs of pages across bitmap words, queues shorter and
+    longer than the workers' window: every result equals the plain path's.
+    (90 PEs x 4096 pages: bitmaps too large for the admitter's shared memory.)"""
+    page = 256
+    arena = arena_pages * page
+    H = (arena + 8 * 64 + 4095) // 4096 * 4096
+    h = heapf(npes, H)
+    lay_amo = arena
+    h.partitions().zero_()
+    rng = np.random.RandomState(count)
+    q = np.zeros(count, sg.REQ_DTYPE)
+    for i in range(count):
+        r = q[i]
+        r["word"], r["flags"] = rng.randint(1, 1 << 60), 1
+        u = rng.rand()
+        if u < 0.6:
+            r["kind"], r["pe"], r["issuer"] = rng.choice([W.OP_PUT, W.OP_GET]), rng.randint(npes), rng.randint(npes)
+            r["n"] = 8 * rng.randint(1, max(2, arena // 2 // 8))
+            r["n"] = min(int(r["n"]), arena // 2 // 16 * 16)
+        elif u < 0.8:
+            r["kind"], r["dtype"], r["flags"], r["word"], r["operand"] = W.OP_FADD, W.DT_INT64, 0, i % 64, 3
+        else:
+            P = rng.randint(1, npes + 1)
+            r["kind"], r["dtype"], r["fmt"], r["issuer"], r["pe"] = W.OP_REDUCE, W.DT_FLOAT, 0xFF, P, rng.randint(npes - P + 1)
+            r["n"] = 4 * rng.randint(1, max(2, arena // 16))
+    cfg = sg.ServerCfg(page_bytes=page, max_inflight=inflight, ring_slots=256, arena_offset=0, arena_bytes=arena, amo_offset=lay_amo, amo_words=64)
+    rec = torch.zeros(sg.COMPLETION_DTYPE.itemsize, dtype=torch.uint8).pin_memory()
+    want = np.zeros(count, np.uint64)
+    for i in range(count):
+        if q[i]["kind"] == W.OP_FADD:
+            continue
+        sg.request_run(q[i:i + 1], cfg, rec.data_ptr())
+        torch.cuda.synchronize()
+        want[i] = rec.numpy().view(sg.COMPLETION_DTYPE)[0]["result"]
+    s = torch.cuda.Stream()
+    srv = sg.Server(cfg, s)
+    recs, got, sent = np.zeros(count, sg.COMPLETION_DTYPE), 0, 0
+    import time
+    end = time.monotonic() + 30
+    try:
+        while got < count and time.monotonic() < end:
+            while sent < count and srv.submit(sg.Req.from_buffer_copy(q[sent].tobytes())) is not None:
+                sent += 1
+            got += srv.poll(recs[got:])
+    finally:
+        srv.stop()
+    assert got == count and not recs["status"].any()
+    order = np.argsort(recs["ticket"], kind="stable")
+    res = recs["result"][order]
+    amo = q["kind"] == W.OP_FADD
+    assert np.array_equal(res[~amo], want[~amo])
+    final = h.view(h.sym(lay_amo), 0, torch.int64, 64).cpu().numpy()
+    for w in range(64):
+        k = np.nonzero(amo & (q["word"] == w))[0]
+        assert sorted(res[k].tolist()) == [3 * j for j in range(len(k))] and final[w] == 3 * len(k)
