@@ -423,7 +423,7 @@ int shmemg_pingpong_cluster(void *buf, uint64_t *sig, uint64_t payload, int npai
  *          rounded up to a multiple of 4 (work space: north and south rows, west and
  *          east columns, each part 16-byte aligned);
  *   sigs   4 uint64, zero before the call (left zero after a successful call).
- * The other tile's contents after the call are unspecified.
+ * The other tile then holds the sweep before the last (with one sweep, the input).
  * shmemg_halo_jacobi: one cooperative launch; after each sweep a PE stores its new
  * boundary rows and columns straight into its four neighbours' halo buffers (device-
  * initiated puts fused into the sweep), then signals each neighbour (put-with-signal,

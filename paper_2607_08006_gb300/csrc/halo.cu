@@ -23,6 +23,8 @@
 // Jacobi update, in this order: out = 0.25 * ((up + down) + (left + right)), binary32 RNE.
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "internal.h"
 
 namespace shmemg {
@@ -418,7 +420,7 @@ __global__ void __launch_bounds__(512) k_halo_prime(HaloArgs a) {
 
 // ------------------------------------------------------------------ tiles held in registers
 // Where a PE's tile fits the registers of its CTAs, the run reads it once, keeps it there
-// for all sweeps and writes it once; a sweep moves only the halos.  A PE is K CTAs here (a
+// for all sweeps and writes the last two states at the end; a sweep moves only the halos.  A PE is K CTAs here (a
 // cluster when K > 1), CTA b holding the row band [ny*b/K, ny*(b+1)/K): thread t owns float4
 // column t mod W4 (W4 = nx/4) and `rpt` consecutive rows of it.  Per sweep a thread publishes
 // its first and last row (and a warp's edge lanes their side columns) in shared memory, one
@@ -434,10 +436,10 @@ __global__ void __launch_bounds__(512) k_halo_prime(HaloArgs a) {
 // reads it, the halo that thread sent after reading it.  Before the first halo a PE zeroes
 // its words and tells its neighbours so with one signal each.
 // What bounds it: about 1 us for the halo's trip and the barriers, and 0.1-0.2 us of
-// instructions per row a thread holds (4.4 us a sweep with 16 rows, 2.3 with 8).  Against the
+// instructions per row a thread holds (4.5 us a sweep with 16 rows, 2.3 with 8).  Against the
 // form that sweeps its tile through L2 (one CTA per PE, 13.7 us a sweep on 64 PEs of 256 x
-// 256): 20 sweeps there 276 -> 89 us, 144 PEs of 128 x 128 155 -> 47 us, one PE of 512 x 512
-// (8 CTAs) 10 sweeps 387 -> 46 us.  Variants measured slower on the first of these: rows
+// 256): 20 sweeps there 276 -> 92 us, 144 PEs of 128 x 128 155 -> 47 us, one PE of 512 x 512
+// (8 CTAs) 10 sweeps 387 -> 48 us.  Variants measured slower on the first of these: rows
 // aligned at the end with branches per row and packed adds (219 us), side columns relayed
 // through shared memory to one word per lane (123 us).
 constexpr int HR_THREADS = 512;
@@ -596,7 +598,7 @@ __global__ void __launch_bounds__(HR_THREADS, 1) k_halo_regs(HaloArgs a, int ite
     const int nprev = b > 0 ? y0 - hr_band(ny, b - 1, K) : 1;
     const int above = (nprev - 1) / ((nprev + R - 1) / R) * W4;
     const bool lsm = live && (lane == 0 || c4 == 0), rsm = live && (lane == 31 || c4 == W4 - 1);
-    for (int t = 0; t < iters; t++) {
+    auto sweep = [&](int t, auto last_sweep) {  // (the last one apart: the others' rows need the registers)
         const int p = t & 1;
         const uint64_t par = (uint64_t)p * words;
         const uint32_t flag = (uint32_t)t + 1;
@@ -627,6 +629,15 @@ __global__ void __launch_bounds__(HR_THREADS, 1) k_halo_regs(HaloArgs a, int ite
                        k < ecnt ? in + part[H_E] + erow + k : nullptr, flag, &s_dead, t, up, dn_end, s_hw + (wrow - y0) + k,
                        s_he + (erow - y0) + k);
         __syncwarp();
+        if (decltype(last_sweep)::value && iters > 1) {
+            // the other tile ends with the sweep before the last, as where the sweeps alternate
+            // between the tiles (tile 1 holds the words: only once every halo has been read)
+            if ((iters & 1) == 0) sync();
+            float *prev = tile0 + (iters & 1 ? 0 : tile_elems);
+#pragma unroll
+            for (int r = 0; r < ROWS; r++)
+                if (live && r < n) *reinterpret_cast<float4 *>(prev + (uint64_t)(i0 + r) * nx + 4 * c4) = v[r];
+        }
         const float *lsrc = west ? s_hw + (i0 - y0) : s_r[p][warp > 0 ? warp - 1 : 0];
         const float *rsrc = east ? s_he + (i0 - y0) : s_l[p][warp < HR_THREADS / 32 - 1 ? warp + 1 : warp];
 #pragma unroll
@@ -648,8 +659,10 @@ __global__ void __launch_bounds__(HR_THREADS, 1) k_halo_regs(HaloArgs a, int ite
                 up = mid;
             }
         }
-        if (t + 1 < iters) send(t + 1);
-    }
+        if (!decltype(last_sweep)::value) send(t + 1);
+    };
+    for (int t = 0; t + 1 < iters; t++) sweep(t, std::false_type());
+    sweep(iters - 1, std::true_type());
     // every halo meant for this PE has been read (the result may lie over the inbox), and no
     // CTA leaves while a peer may still read its rows
     sync();
@@ -683,13 +696,13 @@ static int halo_launch(const void *kernel, void **args, cudaStream_t s) {
 // The register form of a run: CTAs per PE and the kernel, or a null kernel where the tile
 // does not fit: the fewest CTAs that leave a thread at most 8 rows, else at most 16, with every
 // CTA on the GPU at once (more rows per thread cost more than the cluster's barrier: 12 PEs of
-// 400 x 300, 20 sweeps, 59 us against 81 where 16 rows are taken first; 4 rows first gives
+// 400 x 300, 20 sweeps, 63 us against 85 where 16 rows are taken first; 4 rows first gives
 // the same as 8).  Such a run reaches 3-8x the speed of the form below wherever it fits.
 struct HaloRegs {
     const void *kernel;
     int K;
 };
-// (16 full rows spill: 97 us a 64-PE run of 256 x 256 tiles against 89 with the row checks)
+// (16 full rows spill: a 64-PE run of 256 x 256 tiles took 97 us against 89 with the row checks)
 static const void *hr_kernel(int rows, bool full) {
     return rows == 2   ? (full ? (const void *)k_halo_regs<2, true> : (const void *)k_halo_regs<2, false>)
            : rows == 4 ? (full ? (const void *)k_halo_regs<4, true> : (const void *)k_halo_regs<4, false>)

@@ -397,3 +397,27 @@ def test_serving_page_and_slot_reuse(sg, heapf, npes, arena_pages, inflight, cou
     for w in range(64):
         k = np.nonzero(amo & (q["word"] == w))[0]
         assert sorted(res[k].tolist()) == [3 * j for j in range(len(k))] and final[w] == 3 * len(k)
+
+
+@pytest.mark.parametrize("px,py,nx,ny,iters", [(2, 2, 64, 64, 1), (2, 2, 64, 64, 2), (2, 2, 64, 64, 3), (2, 2, 256, 256, 4), (2, 2, 256, 256, 5),
+                                                (3, 1, 132, 61, 7), (1, 1, 2048, 61, 6), (2, 1, 520, 600, 3), (2, 1, 520, 600, 4)])
+def test_halo_other_tile_holds_the_sweep_before(sg, heapf, orc, px, py, nx, ny, iters):
+    """Both tiles after a run -- a second run with odd `iters` starts from what is left in tile 0."""
+    hs, n = sg.halo_stride(nx, ny), nx * ny
+    h = heapf(px * py, (8 * n + 8 * hs + 64 + 4095) // 4096 * 4096)
+    tiles, halos, sigs = h.sym(0, 8 * n), h.sym(8 * n, 8 * hs), h.sym(8 * n + 8 * hs, 32)
+    h.partitions().zero_()
+    grid = W.normals_np(4, px * py * n).astype(np.float32).reshape(py * ny, px * nx)
+    cut = lambda g, p: np.ascontiguousarray(g[p // px * ny:(p // px + 1) * ny, p % px * nx:(p % px + 1) * nx]).reshape(-1)
+    for p in range(px * py):
+        h.view(tiles, p, torch.float32, n).copy_(torch.from_numpy(cut(grid, p)))
+    for run in range(2):
+        sg.halo_jacobi(tiles, halos, sigs, px, py, nx, ny, iters)
+        torch.cuda.synchronize()
+        assert sg.get_status()[0] == 0
+        last, prev = orc.halo_jacobi(grid, iters), orc.halo_jacobi(grid, iters - 1)
+        for p in range(px * py):
+            got = h.view(tiles, p, torch.float32, 2 * n).cpu().numpy().reshape(2, n)
+            assert np.array_equal(got[iters & 1].view(np.uint32), cut(last, p).view(np.uint32))
+            assert np.array_equal(got[(iters & 1) ^ 1].view(np.uint32), cut(prev, p).view(np.uint32))
+        grid = prev if iters & 1 else last
