@@ -454,7 +454,7 @@ typedef struct {
     const float *scales; /* symmetric scales for quantised payloads, else NULL */
 } shmemg_coll_desc_t;
 typedef struct {
-    int32_t tile_elems;   /* elements per work item; 0 = autotune */
+    int32_t tile_elems;   /* elements per work item; 0 = per team, equal shares of the bytes */
     int32_t ctas_per_sm;  /* 0 = occupancy maximum */
     int32_t threads;      /* threads per CTA, 0 = 256 */
     int32_t deep;         /* 0: the kernel held to 3 CTAs per SM; 1: the one held to 2 CTAs

@@ -420,9 +420,10 @@ __global__ void __launch_bounds__(512) k_halo_prime(HaloArgs a) {
 
 // ------------------------------------------------------------------ tiles held in registers
 // Where a PE's tile fits the registers of its CTAs, the run reads it once, keeps it there
-// for all sweeps and writes the last two states at the end; a sweep moves only the halos.  A PE is K CTAs here (a
-// cluster when K > 1), CTA b holding the row band [ny*b/K, ny*(b+1)/K): thread t owns float4
-// column t mod W4 (W4 = nx/4) and `rpt` consecutive rows of it.  Per sweep a thread publishes
+// for all sweeps and writes the last two states at the end; a sweep moves only the halos.  A
+// PE is K CTAs here (a cluster when K > 1), CTA b holding the row band [ny*b/K, ny*(b+1)/K):
+// thread t owns float4 column t mod W4 (W4 = nx/4) and `rpt` consecutive rows of it.  Per
+// sweep a thread publishes
 // its first and last row (and a warp's edge lanes their side columns) in shared memory, one
 // barrier, then updates its rows in place from the top: up and down rows slide in
 // registers, left and right values come from the adjacent lanes; a band's neighbour rows

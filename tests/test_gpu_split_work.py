@@ -421,3 +421,62 @@ def test_halo_other_tile_holds_the_sweep_before(sg, heapf, orc, px, py, nx, ny, 
             assert np.array_equal(got[iters & 1].view(np.uint32), cut(last, p).view(np.uint32))
             assert np.array_equal(got[(iters & 1) ^ 1].view(np.uint32), cut(prev, p).view(np.uint32))
         grid = prev if iters & 1 else last
+
+def test_host_calls_captured_after_joins_and_fills(sg, heapf):
+    """Host-issued calls in a captured stream: after a fill, after a join with another stream, and
+    one after the other; replays give what the calls give."""
+    npes, n = 8, 5003
+    h = heapf(npes, 1 << 17)
+    src, dst, tot, sig = h.malloc(4 * n), h.malloc(4 * n), h.malloc(4 * n), h.malloc(8)
+    x = torch.zeros(n, device="cuda")
+    side = torch.cuda.Stream()
+    g = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(g):
+        x.add_(1.0)
+        h.view(src, 3, torch.float32, n).copy_(x)
+        side.wait_stream(torch.cuda.current_stream())
+        with torch.cuda.stream(side):
+            sg.broadcastmem(sg.TEAM_WORLD, dst, src, 4 * n, 3)
+        torch.cuda.current_stream().wait_stream(side)
+        sg.reduce(sg.TEAM_WORLD, tot, dst, n, sg.FLOAT, sg.SUM)
+        sg.putmem_signal(src, tot, 4 * n, sig, 1, sg.SIGNAL_ADD, 5, 2)
+        sg.atomic("fetch_add", sg.INT64, sig, 10, 5)
+    h.partitions().zero_()
+    torch.cuda.synchronize()
+    for k in range(1, 4):
+        g.replay()
+        torch.cuda.synchronize()
+        assert sg.get_status()[0] == 0
+        for p in range(npes):
+            assert torch.all(h.view(dst, p, torch.float32, n) == float(k))
+            assert torch.all(h.view(tot, p, torch.float32, n) == float(k * npes))
+        assert torch.all(h.view(src, 5, torch.float32, n) == float(k * npes))
+        assert h.view(sig, 5, torch.int64, 1).item() == 11 * k
+
+
+def test_host_calls_chained_on_two_streams(sg, heapf):
+    """A long chain of dependent small calls, handed from one stream to another by events: each
+    sees the whole result of the one before it."""
+    npes = 4
+    h = heapf(npes, 1 << 18)
+    a = h.malloc(40000)
+    h.partitions().zero_()
+    h.view(a, 0, torch.int64, 5000).copy_(torch.arange(5000))
+    s = [torch.cuda.Stream(), torch.cuda.Stream()]
+    for q in s:
+        q.wait_stream(torch.cuda.current_stream())
+    for k in range(200):
+        cur = s[k // 7 % 2]
+        if k % 7 == 0:
+            cur.wait_stream(s[(k // 7 + 1) % 2])
+        if k % 3 == 2:
+            sg.reduce(sg.TEAM_WORLD, a, a, 5000, sg.INT64, sg.MAX, stream=cur)
+        else:
+            sg.putmem(a, a, 40000 - 3 * (k % 2), (k + 1) % npes, k % npes, stream=cur)
+    for q in s:
+        torch.cuda.current_stream().wait_stream(q)
+    sg.reduce(sg.TEAM_WORLD, a, a, 5000, sg.INT64, sg.MAX)
+    want = torch.arange(5000, device="cuda")
+    for p in range(npes):
+        assert torch.equal(h.view(a, p, torch.int64, 5000), want)
