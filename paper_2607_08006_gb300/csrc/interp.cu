@@ -19,7 +19,10 @@
 namespace shmemg {
 
 constexpr int INTERP_THREADS = 512;
-constexpr int OP_BATCH = 64;  // op records staged in shared memory at a time
+// op records staged in shared memory and decoded at a time: 128 (8 KiB) take the common list of an op
+// per PE and a quiet in one go where 64 took two (ring of 64 PEs, 128 KiB each: 12.3 us with 64, 11.4
+// now; a 2000-op script of 4 PEs: 2201 and 2189)
+constexpr int OP_BATCH = 128;
 // shared-team alltoalls staged through the DSMEM windows: at most this many bytes per
 // member (P blocks).  Measured on a cluster of 8 PEs: staged 3.96 / 4.48 / 4.91 us per op
 // at 64 B / 512 B / 1 KiB blocks against 5.53-5.58 us through L2, and behind from 2 KiB
@@ -274,8 +277,9 @@ __device__ __forceinline__ void mb_set(uint64_t *p, uint32_t epoch, uint32_t n) 
 // after each one.  Waits are bounded: a load that never lands ends the lean loop with a
 // timeout (status set); the ring is then left alone and later transfers are counted done
 // without being moved, so no quiet waits forever.  An agent that sees no post, no new op
-// batch of its PE and no exit flag for 8 x timeout_ns (longer than any bounded wait of the
-// PE) records a timeout (detail -5) and leaves; a later quiet on it then times out in the PE.
+// batch of its PE and no exit flag for 16 x timeout_ns (an eighth of a batch's
+// ops, were each to wait its full bound) records a timeout (detail -5) and leaves; a later
+// quiet on it then times out in the PE.
 __device__ __noinline__ void ctx_agent(const shmemg_device_ctx_t &c, CtxMailbox *mb, uint32_t epoch, uint8_t *ring,
                                        uint64_t *bars) {
     uint32_t taken[NQ - 1] = {}, beat = 0, nap = 128;
@@ -310,7 +314,7 @@ __device__ __noinline__ void ctx_agent(const shmemg_device_ctx_t &c, CtxMailbox 
         const uint64_t now = shmemg_d_globaltimer();
         const uint32_t b = *(volatile uint32_t *)&mb->beat;
         if (idle_since == 0 || b != beat) idle_since = now, beat = b;
-        else if (now - idle_since > 8 * c.timeout_ns) {
+        else if (now - idle_since > OP_BATCH / 8 * c.timeout_ns) {
             shmemg_d_set_status(c, SHMEMG_ERR_TIMEOUT, -5);
             break;
         }
@@ -441,7 +445,7 @@ constexpr int OP_WINDOW = 7;                 // ops since the last PE barrier th
 constexpr uint32_t OP_APART = 0x80u, OP_OWN_SYNC = OP_APART;  // not simple; and no barrier before it
 
 // Warp 0, per batch: conf of the listed ops -- bit d - 1: the op conflicts with the listed op d
-// before it (all of the first half of the batch conflict with the second).  Ranges are compared
+// before it (the last ops of one 32 conflict with the first of the next).  Ranges are compared
 // in granules of 2^gran bytes over the whole heap, which fit 32 bits; branch-free (this code
 // runs cold in a short script: a switch's jump table cost it half a microsecond).
 __device__ __forceinline__ void op_conflicts(const shmemg_op_t *ops, const uint8_t *act, const uint8_t *list, uint8_t *conf,
@@ -591,7 +595,13 @@ __global__ void __launch_bounds__(INTERP_THREADS, 1) k_interp(shmemg_device_ctx_
         }
         if (lane == 0) s_nact = nact;
         __syncwarp();
-        op_conflicts(s_ops, s_act, s_list, s_conf, nact, c.pe_stride, gran);
+        // (nothing to compare a single op with: many PEs with short lists skip the code's cold fetch)
+        if (nact > 1) {
+            op_conflicts(s_ops, s_act, s_list, s_conf, nact, c.pe_stride, gran);
+        } else if (nact == 1 && lane == 0) {
+            const int k = s_list[0];
+            s_conf[0] = s_act[k] == 1 && s_ops[k].kind - SHMEMG_OP_BARRIER_ALL < 3u ? (uint8_t)OP_OWN_SYNC : (uint8_t)0;
+        }
     }
     __syncthreads();
     if (dma && dma_busy(s_dma)) dma_progress(s_dma, s_ring);  // background transfers advance

@@ -311,6 +311,31 @@ def test_script_ops_of_one_pe_keep_their_order(sg, heapf, orc, mode, cd, span, b
         assert np.array_equal(fetched.cpu().numpy()[amo], np.asarray(want)[amo])
 
 
+@pytest.mark.parametrize("mode,cd", [(0, 1), (1, 2)])
+@pytest.mark.parametrize("n", [8, 4096, 131072])
+@pytest.mark.parametrize("at", [126, 127, 128, 255])
+def test_script_op_alone_in_its_batch_sees_the_one_before(sg, heapf, orc, mode, cd, n, at):
+    """PE 0 has two ops, at the end of one batch of the list and alone in the next (or beside it): a
+    put, and a get of what it wrote."""
+    npes, H = 3, 1 << 19
+    ops = np.zeros(at + 2, W.OP_DTYPE)
+    ops["kind"], ops["dtype"], ops["issuer"], ops["pe"] = W.OP_FADD, W.DT_INT64, 2, 2
+    ops["dst"], ops["operand"] = 8 * (np.arange(at + 2) % 16), 3
+    for i, kind, dst, src in ((at, W.OP_PUT, 1 << 17, 0), (at + 1, W.OP_GET, 2 << 17, 1 << 17)):
+        ops[i] = np.zeros(1, W.OP_DTYPE)[0]
+        ops[i]["kind"], ops[i]["issuer"], ops[i]["pe"], ops[i]["n"], ops[i]["dst"], ops[i]["src"] = kind, 0, 1, n, dst, src
+    h = heapf(npes, H, pe_mode=mode, cluster_dim=cd)
+    init = random_heap(npes, H, at)
+    upload(h, init)
+    fetched = torch.zeros(len(ops), dtype=torch.int64, device="cuda")
+    sg.run_script(torch.from_numpy(ops.view(np.uint8).copy()).cuda(), len(ops), fetched)
+    torch.cuda.synchronize()
+    assert sg.get_status()[0] == 0
+    ref = orc.Heap(npes, H, init)
+    ref.run_script(ops)
+    assert first_diff(download(h), ref.mem) is None
+
+
 @pytest.mark.parametrize("npes", [1, 2, 5, 64])
 def test_barriers_back_to_back(sg, heapf, orc, npes):
     """Consecutive barriers, in which PEs arrive at the next before the last has been folded:
