@@ -757,7 +757,10 @@ __global__ void __launch_bounds__(INTERP_THREADS, 1) k_interp(shmemg_device_ctx_
                 } else if (dma && ctx_home && o.sub != 0) {
                     dma_drain(c, s_dma, s_ring, o.sub == SHMEMG_CTX_ALL ? -1 : o.sub);
                 }
-                shmemg_d_quiet_pe(c);
+                // every thread fences after the PE barrier: whichever issues a later op (small
+                // ones start on any warp) orders it itself after all the PE's earlier ones
+                shmemg_d_pe_sync(c);
+                shmemg_d_fence_gpu();
             }
             break;
         case SHMEMG_OP_BARRIER_ALL:
