@@ -439,8 +439,11 @@ __device__ __forceinline__ bool op_involves(const shmemg_op_t &o, int me) {
 
 // Which of a PE's ops need a PE barrier before them.  Consecutive puts, gets and AMOs (PE scope;
 // non-blocking ones on the default context) need none between them unless one touches what
-// another writes; every other op is kept apart, but those that begin with a PE barrier of
-// their own -- quiet, fence, barrier_all, the world team's collectives -- need none before.
+// another writes.  put_signal ends with the leader's update of the signal word, after the PE barrier
+// that closes its own copy and all before it: what it leaves open is that word.  Every other op
+// is kept apart, but those that begin with a PE barrier of their own -- quiet, fence, barrier_all,
+// the world team's collectives -- need none before, nor does a wait after put_signals (both are
+// the leader's).
 constexpr int OP_WINDOW = 7;                 // ops since the last PE barrier that an op is checked against
 constexpr uint32_t OP_APART = 0x80u, OP_OWN_SYNC = OP_APART;  // not simple; and no barrier before it
 
@@ -457,7 +460,8 @@ __device__ __forceinline__ void op_conflicts(const shmemg_op_t *ops, const uint8
         const shmemg_op_t &o = ops[at];
         const uint32_t k = o.kind;  // (flags in it: a warp-scope op is not simple)
         const bool valid = in && act[at] == 1, nbi = k == SHMEMG_OP_PUT_NBI || k == SHMEMG_OP_GET_NBI;
-        const bool amo = k - SHMEMG_OP_FETCH_ADD < 3u, put = k == SHMEMG_OP_PUT || k == SHMEMG_OP_PUT_NBI;
+        const bool amo = k - SHMEMG_OP_FETCH_ADD < 3u, psig = valid && k == SHMEMG_OP_PUT_SIGNAL;
+        const bool put = k == SHMEMG_OP_PUT || k == SHMEMG_OP_PUT_NBI || psig;
         const bool simple = valid && k - SHMEMG_OP_PUT < 7u && !(nbi && o.sub != 0);
         const bool own = valid && (k - SHMEMG_OP_BARRIER_ALL < 3u || (k - SHMEMG_OP_BROADCAST < 5u && o.team == SHMEMG_TEAM_WORLD));
         const uint64_t there = (uint64_t)o.pe * H, mine = (uint64_t)o.issuer * H, n = amo ? 8 : o.n;
@@ -465,15 +469,23 @@ __device__ __forceinline__ void op_conflicts(const shmemg_op_t *ops, const uint8
         // first and last granule (an empty range touches its first)
         const uint32_t w0 = (uint32_t)(w >> gran), w1 = (uint32_t)((w + (n ? n - 1 : 0)) >> gran);
         const uint32_t r0 = (uint32_t)(r >> gran), r1 = (uint32_t)((r + (n ? n - 1 : 0)) >> gran);
+        // what the op leaves open to those after it
+        const uint32_t sig = (uint32_t)((there + o.aux) >> gran);
+        const uint32_t ow0 = psig ? sig : w0, ow1 = psig ? sig : w1, or0 = psig ? sig : r0, or1 = psig ? sig : r1;
+        const uint32_t psigs = __ballot_sync(0xffffffffu, psig), after_psig = __brev((psigs << 1) << (31 - lane));
         const int most = nact - k0 - 1 < OP_WINDOW ? nact - k0 - 1 : OP_WINDOW;
-        uint32_t m = simple ? 0u : own ? OP_OWN_SYNC : 0xFFu;
+        uint32_t hits = 0;
         for (int d = 1; d <= most; d++) {
-            const uint32_t q0 = __shfl_up_sync(0xffffffffu, r0, d), q1 = __shfl_up_sync(0xffffffffu, r1, d);
-            const uint32_t v0 = __shfl_up_sync(0xffffffffu, w0, d), v1 = __shfl_up_sync(0xffffffffu, w1, d);
-            if (simple && lane >= d && ((r0 <= v1 && v0 <= r1) || (w0 <= v1 && v0 <= w1) || (w0 <= q1 && q0 <= w1))) m |= 1u << (d - 1);
+            const uint32_t q0 = __shfl_up_sync(0xffffffffu, or0, d), q1 = __shfl_up_sync(0xffffffffu, or1, d);
+            const uint32_t v0 = __shfl_up_sync(0xffffffffu, ow0, d), v1 = __shfl_up_sync(0xffffffffu, ow1, d);
+            if ((r0 <= v1 && v0 <= r1) || (w0 <= v1 && v0 <= w1) || (w0 <= q1 && q0 <= w1)) hits |= 1u << (d - 1);
         }
+        hits &= (1u << lane) - 1u;
+        // a put_signal: every op before it but put_signals that it does not touch; a wait: every op but
+        // put_signals
+        uint32_t m = simple ? hits : own ? 0u : psig ? (hits | ~after_psig) & 0x7Fu : k == SHMEMG_OP_WAIT_UNTIL && valid ? ~after_psig & 0x7Fu : 0x7Fu;
         if (k0 > 0 && lane < OP_WINDOW && !own) m |= (0xFFu << lane) & 0x7Fu;
-        if (in) conf[k0 + lane] = (uint8_t)m;
+        if (in) conf[k0 + lane] = (uint8_t)(simple || psig ? m : m | OP_APART);
     }
 }
 
@@ -621,7 +633,7 @@ __global__ void __launch_bounds__(INTERP_THREADS, 1) k_interp(shmemg_device_ctx_
                 q_sync = qi;
                 carry = false;
             }
-            if (conf & OP_APART) q_sync = qi + 1, carry = false;  // (begins or ends with a PE barrier, or completes at a quiet)
+            if (conf & OP_APART) q_sync = qi + 1, carry = false;  // (ends with a PE barrier, or completes at a quiet)
             k = s_list[qi++];
         } else {
             if (!dsm || k_next >= cnt) break;

@@ -5,7 +5,7 @@ import pytest
 import torch
 
 import workloads as W
-from gpu_util import random_heap, upload
+from gpu_util import download, first_diff, random_heap, upload
 
 pytestmark = pytest.mark.gpu
 KiB = 1 << 10
@@ -75,3 +75,48 @@ def test_flag_after_quiet_or_fence_follows_the_data(sg, heapf, mode, cd, order, 
         for r in range(rounds):
             src = SRC + 16 * r if n > 8 else SRC + 8 * r
             assert np.array_equal(got[r], m[0, src:src + n]), r
+
+
+@pytest.mark.parametrize("mode,cd", [(0, 1), (1, 2)])
+@pytest.mark.parametrize("sig", [0, 1])
+@pytest.mark.parametrize("seed", [1, 2])
+@pytest.mark.parametrize("pad", [0, 125, 126, 127])
+def test_ops_on_the_signal_word_follow_the_signal(sg, heapf, orc, mode, cd, sig, seed, pad):
+    """put_signal, then by the same PE an AMO, a put, a get or another put_signal that reads or writes the
+    signal word: the list's result, also across the end of a batch of the list."""
+    npes, H = 3, 1 << 18
+    rng = np.random.RandomState(seed)
+    SIG, DATA, TMP = 64 * KiB, 0, 128 * KiB
+    ops = [_rec(kind=W.OP_FADD, dtype=W.DT_INT64, issuer=2, pe=2, dst=8 * (i % 16), operand=3) for i in range(pad)]
+    for r in range(120):
+        to, w = rng.randint(0, npes), SIG + 8 * rng.randint(0, 2)
+        put = dict(kind=W.OP_PUT_SIGNAL, sub=sig, issuer=0, pe=to, aux=w, operand=5 + r)
+        # (a put before it turns the ops that follow to other threads)
+        ops.append(_rec(kind=W.OP_PUT, issuer=0, pe=1, dst=TMP, src=DATA, n=8 * rng.randint(1, 600)))
+        ops.append(_rec(**put, dst=192 * KiB, src=DATA, n=int(rng.choice([0, 8, 4096, 40000]))))
+        u = r % 5
+        if u == 0:
+            ops.append(_rec(kind=W.OP_FADD, dtype=W.DT_INT64, issuer=0, pe=to, dst=w, operand=1 << 20))
+        elif u == 1:
+            ops.append(_rec(kind=W.OP_PUT, issuer=0, pe=to, dst=w, src=DATA + 8 * (r % 64), n=8))
+        elif u == 2:
+            ops.append(_rec(kind=W.OP_GET, issuer=0, pe=to, dst=TMP + 32 * KiB + 8 * r, src=w, n=8))
+        elif u == 3:  # another put_signal that carries the word
+            ops.append(_rec(kind=W.OP_PUT_SIGNAL, sub=sig, issuer=0, pe=2, aux=SIG + 32, operand=1, dst=TMP + 48 * KiB + 8 * r, src=w, n=8)
+                       if to == 0 else _rec(**put, dst=w, src=DATA + 8, n=8))
+        else:
+            ops.append(_rec(kind=W.OP_FXOR, dtype=W.DT_INT64, issuer=0, pe=to, dst=w, operand=r))
+            ops.append(_rec(kind=W.OP_GET, issuer=0, pe=to, dst=TMP + 32 * KiB + 8 * r, src=SIG, n=16))
+    ops_np, dev = _dev(ops)
+    h = heapf(npes, H, pe_mode=mode, cluster_dim=cd)
+    init = random_heap(npes, H, seed)
+    upload(h, init)
+    fetched = torch.zeros(len(ops), dtype=torch.int64, device="cuda")
+    sg.run_script(dev, len(ops), fetched)
+    torch.cuda.synchronize()
+    assert sg.get_status()[0] == 0
+    ref = orc.Heap(npes, H, init)
+    want = ref.run_script(ops_np)
+    assert first_diff(download(h), ref.mem) is None
+    amo = np.isin(ops_np["kind"], [W.OP_FADD, W.OP_FXOR])
+    assert np.array_equal(fetched.cpu().numpy()[amo], np.asarray(want)[amo])
