@@ -35,14 +35,24 @@ __device__ __forceinline__ uint2 q_encode(uint64_t lo, uint64_t hi) {
 // quotient.  y moved by 2^-21 down and up (and by the two products' own 2^-24) therefore
 // encloses the quotient, and encoding is monotonic: where both ends have the same code, that is
 // the quotient's.  The ends differ for about one element in 2^16 (E4M3) or 2^12 (bf16).  `safe`: s and
-// 1/s far from the ends of binary32's range, so that r is that exact; results below the
-// normal range are too small for either format's first code (both ends give zero).
+// 1/s far from the ends of binary32's range, so that r is that exact.  Products near or below the
+// normal range (2^-126) keep fewer bits than that.  E4M3's first code is far above them: both ends
+// give zero, and so does the quotient.  bf16's is 2^-133: a non-zero product below 2^-120 takes
+// the divisions (one that rounds to zero is below 2^-149, and its code zero either way).
 template <int FMT>
 __device__ __forceinline__ uint2 q_codes(const float (&v)[4], float s, float r, bool safe) {
     const uint64_t rr = f2(r, r), dn = f2(1.0f - 0x1p-21f, 1.0f - 0x1p-21f), up = f2(1.0f + 0x1p-21f, 1.0f + 0x1p-21f);
     const uint64_t y0 = f2_mul(f2(v[0], v[1]), rr), y1 = f2_mul(f2(v[2], v[3]), rr);
     const uint2 a = q_encode<FMT>(f2_mul(y0, dn), f2_mul(y1, dn)), b = q_encode<FMT>(f2_mul(y0, up), f2_mul(y1, up));
-    if (safe && a.x == b.x && a.y == b.y) return a;
+    safe = safe && a.x == b.x && a.y == b.y;
+    if (FMT == SHMEMG_FMT_E4M3) {
+        if (safe) return a;
+    } else {
+        const float least = fminf(fminf(fabsf(f2_lo(y0)), fabsf(f2_hi(y0))), fminf(fabsf(f2_lo(y1)), fabsf(f2_hi(y1))));
+        if (safe && least >= 0x1p-120f) return a;
+        auto low = [](float y) { return y != 0.0f && fabsf(y) < 0x1p-120f; };
+        if (safe && !(low(f2_lo(y0)) || low(f2_hi(y0)) || low(f2_lo(y1)) || low(f2_hi(y1)))) return a;
+    }
     return q_encode<FMT>(f2(__fdiv_rn(v[0], s), __fdiv_rn(v[1], s)), f2(__fdiv_rn(v[2], s), __fdiv_rn(v[3], s)));
 }
 

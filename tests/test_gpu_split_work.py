@@ -201,6 +201,38 @@ def test_quantize_near_the_midpoints(sg, heapf, orc, fmt, n, qshift):
         assert np.array_equal(gq, np.asarray(wq).view(np.uint8).reshape(-1))
 
 
+@pytest.mark.parametrize("n,qshift", [(128 * 96, 0), (128 * 95 + 77, 1)])
+def test_quantize_bf16_below_the_normal_range(sg, heapf, orc, n, qshift):
+    """Quotients near the midpoints of bf16's subnormal codes, which binary32 holds with few bits: the
+    code is the division's."""
+    rng = np.random.RandomState(17)
+    x = np.zeros((2, 96 * 128), np.float32)
+    for p in range(2):
+        for b in range(96):
+            amax = np.float32(np.ldexp(1 + rng.rand(), rng.randint(-3, 101)))
+            q = (rng.randint(0, 0x101, 128) + 0.5 + rng.randint(-3, 4, 128) * 2.0 ** -16) * 2.0 ** -133
+            with np.errstate(under="ignore"):
+                v = (q * rng.choice([-1.0, 1.0], 128) * np.float64(amax)).astype(np.float32)
+            v[0] = amax
+            x[p, 128 * b:128 * b + 128] = v
+    # pairs whose product with the reciprocal lies on the other side
+    x[0, 0:2] = np.array([0x3f81f780, 0x000fbcf8], np.uint32).view(np.float32)
+    x[0, 2:128] = 0.0
+    x[0, 128:130] = [float.fromhex("0x1.25a05cp+85"), float.fromhex("0x1.4a548cp-46")]
+    h = heapf(2, 1 << 18)
+    src, sc, q = h.malloc(4 * n), h.malloc(4 * 96), h.malloc(2 * (n + 8))
+    for p in range(2):
+        h.view(src, p, torch.float32, n).copy_(torch.from_numpy(x[p, :n]))
+    sg.quantize(sg.TEAM_WORLD, q.ptr + 2 * qshift, sc, src, 0, n)
+    torch.cuda.synchronize()
+    for p in range(2):
+        wq, ws = orc.quantize(x[p, :n], 0)
+        gs = h.view(sc, p, torch.float32, len(ws)).cpu().numpy()
+        gq = h.view(h.sym(q.offset + 2 * qshift), p, torch.uint16, n).cpu().numpy()
+        assert np.array_equal(gs.view(np.uint32), np.asarray(ws, np.float32).view(np.uint32))
+        assert np.array_equal(gq, np.asarray(wq).view(np.uint16).reshape(-1))
+
+
 @pytest.mark.parametrize("fmt", [0, 1])
 @pytest.mark.parametrize("P,n,shift", [(1, 1, 0), (3, 1023, 0), (8, 1024, 0), (17, 5121, 0), (5, 2000, 1), (2, 2 * 608 * 2048 + 1029, 0)])
 def test_qsum_chunk_forms(sg, heapf, orc, fmt, P, n, shift):
