@@ -18,6 +18,7 @@
 #include <cuda_runtime.h>
 #include <time.h>
 
+#include <cstddef>
 #include <cstring>
 #include <thread>
 
@@ -75,7 +76,7 @@ struct __align__(128) SvSlot {
     shmemg_req_t req;
     uint64_t dst_off;
     uint32_t page0, npages;
-    uint32_t ntiles, gen;
+    uint32_t ntiles, gen;            // (one aligned 64-bit word: written and read together)
     uint64_t t_admit;
     uint64_t t_pub;                  // when the admitter queued it
     int32_t status;
@@ -90,6 +91,10 @@ struct __align__(128) SvSlot {
     uint8_t pad3[112];
 };
 static_assert(sizeof(SvSlot) == 384, "slot layout");
+static_assert(offsetof(SvSlot, ntiles) % 8 == 0 && offsetof(SvSlot, gen) == offsetof(SvSlot, ntiles) + 4, "slot layout");
+
+// a slot's tile count (low half) with the generation it belongs to
+__device__ __forceinline__ uint64_t slot_tiles(const SvSlot &s) { return *(const volatile uint64_t *)&s.ntiles; }
 
 struct SvArgs {
     uint8_t *heap;
@@ -704,8 +709,7 @@ __device__ int adm_try(const SvArgs &a, AdmState &st, unsigned long long *sh, un
         s.dst_off = a.cfg.arena_offset + (uint64_t)p0 * a.cfg.page_bytes;
         s.page0 = p0;
         s.npages = need;
-        s.ntiles = g.ntiles;
-        s.gen = gen;
+        *(volatile uint64_t *)&s.ntiles = (uint64_t)g.ntiles | ((uint64_t)gen << 32);
         s.t_admit = now;
         s.status = 0;
         s.busy = 1;
@@ -867,9 +871,10 @@ __device__ __forceinline__ bool publish(const SvArgs &a, uint32_t slot, uint64_t
 // chunk size on the slot's (generation, next tile) word with acquire semantics (the
 // admitter published the slot with a release store of that word).  Big requests are
 // claimed in chunks (about half of an even share per worker), so the claim word and
-// the completion counter see few atomics; a claimed index below ntiles is always
-// executed, even by a worker that came from an older queue entry of the same slot, so
-// no index is lost.
+// the completion counter see few atomics; a claimed index below the tile count of the
+// generation it was claimed from is always executed, even by a worker that came from an older
+// queue entry of the same slot, so no index is lost.  An index claimed from an exhausted
+// request is dropped, also where the slot holds another by the time its tile count is read.
 __device__ __forceinline__ bool claim_tiles(const SvArgs &a, uint32_t slot, uint32_t *tile, uint32_t *cnt,
                                             shmemg_req_t *req, uint64_t *dst_off, uint32_t *nstage,
                                             uint32_t nt_seen = 0) {
@@ -886,11 +891,12 @@ __device__ __forceinline__ bool claim_tiles(const SvArgs &a, uint32_t slot, uint
                  : "memory");
     // the request and its destination are read together with the tile count (all ordered
     // after the acquire above), so the claim costs one round trip more, not three
-    const uint32_t k = (uint32_t)c, n = *(volatile uint32_t *)&s.ntiles;
+    const uint64_t tiles = slot_tiles(s);
+    const uint32_t k = (uint32_t)c, n = (uint32_t)tiles;
     const shmemg_req_t rq = s.req;
     const uint64_t d = s.dst_off;
     const uint32_t ns = s.nstage;
-    if (k < n) {
+    if (k < n && (uint32_t)(tiles >> 32) == (uint32_t)(c >> 32)) {
         *tile = k;
         *cnt = k + chunk <= n ? chunk : n - k;
         *req = rq;
