@@ -697,6 +697,7 @@ __device__ int adm_try(const SvArgs &a, AdmState &st, unsigned long long *sh, un
             ok = shmemg_d_ld_acquire_u32(&a.slots[k].busy) == 0;
         }
         st.slot_free = __ballot_sync(0xffffffffu, ok);
+        __syncwarp();  // (the lanes that write a slot come after the one that saw it free)
     }
     uint32_t p0 = 0;
     if (!take_pages(a, sh, g, need, &p0, lane)) return 0;
@@ -1000,8 +1001,9 @@ __device__ void worker(const SvArgs &a) {
                     cmd = go;
                     break;
                 }
-                h = __shfl_sync(0xffffffffu, h, 0);  // (orders the other lanes' reads after the acquires)
+                h = __shfl_sync(0xffffffffu, h, 0);
                 t = __shfl_sync(0xffffffffu, t, 0);
+                __syncwarp();  // the other lanes' reads come after lane 0's acquires (a shuffle orders no memory)
                 const uint32_t live = (uint32_t)((t - h) < WINDOW ? (t - h) : WINDOW);
                 const bool valid = (uint32_t)lane < live;
                 const unsigned long long e = valid ? *(volatile unsigned long long *)&a.fifo[(h + lane) % a.fifo_cap] : 0ull;
