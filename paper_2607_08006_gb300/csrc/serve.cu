@@ -856,16 +856,17 @@ __device__ void finalize(const SvArgs &a, SvSlot &s, int lane) {
 // Publishes `cnt` finished tiles of slot s with their checksum terms (AMO: the fetched
 // value): one acq_rel add on the tile count -- release for this CTA's tile writes
 // (ordered before it by a CTA barrier) and the checksum, acquire for the other
-// publishers'.  True for the publisher that completes the count (it finalizes).
+// publishers'.  True for the publisher that completes the count (it finalizes).  The tile count
+// is read before the add: after it the slot may already hold another request.
 __device__ __forceinline__ bool publish(const SvArgs &a, uint32_t slot, uint64_t sum, unsigned long long amo,
                                         uint32_t cnt) {
     SvSlot &s = a.slots[slot];
-    const uint32_t kind = s.req.kind;
+    const uint32_t kind = s.req.kind, ntiles = *(volatile uint32_t *)&s.ntiles;
     if (kind == SHMEMG_OP_FETCH_ADD || kind == SHMEMG_OP_COMPARE_SWAP || kind == SHMEMG_OP_FETCH_XOR) s.checksum = amo;
     else atomicAdd(&s.checksum, (unsigned long long)sum);
     unsigned int old;
     asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(&s.done), "r"(cnt) : "memory");
-    return old + cnt == s.ntiles;
+    return old + cnt == ntiles;
 }
 
 // Claims tiles [k, k + cnt) of whatever request slot s holds now: fetch-and-add of the
