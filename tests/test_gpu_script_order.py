@@ -120,3 +120,29 @@ def test_ops_on_the_signal_word_follow_the_signal(sg, heapf, orc, mode, cd, sig,
     assert first_diff(download(h), ref.mem) is None
     amo = np.isin(ops_np["kind"], [W.OP_FADD, W.OP_FXOR])
     assert np.array_equal(fetched.cpu().numpy()[amo], np.asarray(want)[amo])
+
+
+def test_agent_gives_a_silent_pe_eight_timeouts(sg, heapf):
+    """A context agent whose PE shows no sign of life -- here during a short list of long puts --
+    reports a timeout after eight of them and not after five."""
+    H, n, count = 1 << 30, 256 << 20, 48
+    h = heapf(2, H)
+    ops = [_rec(kind=W.OP_PUT, issuer=0, pe=1, dst=512 << 20, src=0, n=n) for _ in range(count)]
+    _, dev = _dev(ops)
+    t = []
+    for _ in range(2):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        sg.run_script(dev, count, None)
+        b.record()
+        torch.cuda.synchronize()
+        t.append(a.elapsed_time(b) * 1e6)
+    assert sg.get_status()[0] == 0
+    h.close()
+    for parts, want in ((5, 0), (12, sg.ERR_TIMEOUT)):
+        h = heapf(2, H, timeout_ns=int(t[1] / parts))
+        sg.run_script(dev, count, None)
+        torch.cuda.synchronize()
+        status, detail = sg.get_status()
+        assert status == want and (status == 0 or detail == -5), (parts, status, detail)
+        h.close()
