@@ -466,8 +466,8 @@ typedef struct shmemg_batch_s *shmemg_batch_t;
 int shmemg_batch_create(const shmemg_coll_desc_t *descs, int count, const shmemg_tune_t *tune,
                         shmemg_batch_t *out);
 int shmemg_batch_launch(shmemg_batch_t batch, void *stream);
-/* Times each candidate plan with CUDA events on `stream`, keeps the fastest, re-captures
- * the graph, and reports the choice in *chosen (may be NULL). */
+/* Times each candidate plan, the batch's own among them, with CUDA events on `stream`, keeps
+ * the fastest, re-captures the graph, and reports the choice in *chosen (may be NULL). */
 int shmemg_batch_autotune(shmemg_batch_t batch, void *stream, shmemg_tune_t *chosen);
 int shmemg_batch_destroy(shmemg_batch_t batch);
 

@@ -201,6 +201,28 @@ def test_quantize_near_the_midpoints(sg, heapf, orc, fmt, n, qshift):
         assert np.array_equal(gq, np.asarray(wq).view(np.uint8).reshape(-1))
 
 
+def test_autotune_keeps_the_batch_s_own_plan_where_it_is_the_fastest(sg, heapf):
+    """Four teams of 128 PEs x 8192 int64: the uniform tiles leave most of the GPU idle (three times the
+    per-team plan's time)."""
+    P, n = 128, 8192
+    h = heapf(P, 8 * 8 * n + 65536)
+    objs = [(h.malloc(8 * n), h.malloc(8 * n)) for _ in range(4)]
+    x = torch.arange(n, device="cuda")
+    for k, (_, src) in enumerate(objs):
+        for p in range(P):
+            h.view(src, p, torch.int64, n).copy_(x * (k + 1) + p)
+    b = sg.Batch([sg.CollDesc(0, P, sg.INT64, -1, n, dst.ptr, src.ptr, None) for dst, src in objs], None)
+    assert b.autotune().tile_elems == 0
+    for dst, _ in objs:
+        for p in range(P):
+            h.view(dst, p, torch.int64, n).zero_()
+    b.launch()
+    for k, (dst, _) in enumerate(objs):
+        for p in (0, 77, P - 1):
+            assert torch.equal(h.view(dst, p, torch.int64, n), x * (k + 1) * P + P * (P - 1) // 2)
+    b.destroy()
+
+
 @pytest.mark.parametrize("n,qshift", [(128 * 96, 0), (128 * 95 + 77, 1)])
 def test_quantize_bf16_below_the_normal_range(sg, heapf, orc, n, qshift):
     """Quotients near the midpoints of bf16's subnormal codes, which binary32 holds with few bits: the
