@@ -771,8 +771,12 @@ extern "C" int shmemg_halo_jacobi(float *tiles, float *halos, uint64_t *sigs, in
     // tiles of more than two rows sweep their interior while the halos are on the way; where
     // the heap's PEs are single CTAs and the GPU holds several per PE, a PE is a cluster of
     // them here (the sweep splits its tile over a PE's threads either way): 64 PEs of 512 x
-    // 512, 10 sweeps, 407 -> 274 us with two CTAs each, two of 1024 x 1024 1364 -> 230 with eight
-    if (ny > 2 && st().pe_mode == SHMEMG_PE_MODE_CTA && st().cluster_dim == 1)
+    // 512, 10 sweeps, 407 -> 274 us with two CTAs each, two of 1024 x 1024 1364 -> 230 with eight.
+    // A tile of less than two float4 a thread of one CTA stays with one, whose barrier is the
+    // cheaper (20 sweeps of 4 PEs: 8 x 8 87 us against 98 with eight, 16 x 15 91 and 106, 256 x 6 86
+    // and 106, 4 x 512 115 and 120, 8 x 64 98 and 102, 4 x 64 108 and 105; 1024 x 4 119 and 109,
+    // 4 x 1024 136 and 120)
+    if (ny > 2 && (int64_t)nx * ny >= 2 * 4 * 512 && st().pe_mode == SHMEMG_PE_MODE_CTA && st().cluster_dim == 1)
         for (int K = 8; K > 1; K /= 2) {
             const void *kf = (const void *)k_halo<true>;
             if (halo_smem_granted(kf, 512) &&

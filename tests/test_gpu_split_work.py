@@ -34,6 +34,14 @@ def test_halo_tiles_in_registers(sg, heapf, orc, px, py, nx, ny, iters):
     assert not sig.any()
 
 
+@pytest.mark.parametrize("px,py,nx,ny", [(2, 2, 8, 8), (1, 1, 4, 3), (2, 1, 4, 1023), (2, 1, 4, 1024), (1, 2, 1020, 4), (1, 2, 1024, 4)])
+def test_halo_tiles_too_thin_for_registers(sg, heapf, orc, px, py, nx, ny):
+    """Streamed tiles on either side of 4096 points, from which several CTAs take a PE."""
+    got, want, sig = _run_halo(sg, heapf, orc, px, py, nx, ny, 5)
+    assert np.array_equal(got.view(np.uint32), want.view(np.uint32))
+    assert not sig.any()
+
+
 @pytest.mark.parametrize("nx,ny", [(64, 64), (256, 200)])
 def test_halo_captured_and_replayed(sg, heapf, orc, nx, ny):
     """A captured run (one CTA per PE; several) replays on what the last replay left."""
