@@ -34,11 +34,11 @@ struct AmoArgs {
 // left 88 of 152 SMs idle on a 64-PE heap (4 Mi random ops on a 128 MiB table: 294 us, now
 // 115; 1 Mi ops on an 8 MiB one: 45.1 us, now 12.3).  A random atomic is bound by
 // the rate of the table's sector fills and write-backs once enough are in flight, and more
-// lower it: with 6 CTAs per SM and 4 atomics per thread 4 Mi ops on a 512 MiB table ran
-// 150 us against 140 with 3 and 2 (the 128 MiB table 112 against 109; tables inside the L2
-// the same), so a plain stream runs AMO_PLAIN_CTAS CTAs per SM.  The aggregating form
-// has one pass of a warp in flight at a time and takes every CTA that fits (289 against
-// 284 us, 4 M Zipf ops).
+// lower it: with 6 CTAs per SM and 4 atomics per thread 4 Mi ops on 1024 PEs' 512 MiB table
+// run 177.6 us against 164.5 with 3 and 2, on 64 PEs' 128 MiB table 103.6 against 99.8 (32 MiB
+// 67.4 and 68.6, 8 MiB 11.2 and 11.1), so a plain stream runs AMO_PLAIN_CTAS CTAs per SM.  The
+// aggregating form has one pass of a warp in flight at a time and takes every CTA that fits: 4 M
+// Zipf ops on 16 PEs 94.9 us, 98.4 with 3 per SM.
 constexpr int AMO_U = 2;  // atomics in flight per thread
 constexpr int AMO_PLAIN_CTAS = 3;
 __global__ void __launch_bounds__(AMO_THREADS, 6) k_amo_stream(AmoArgs a) {
